@@ -164,13 +164,13 @@ __device__ __forceinline__ void block_sum_batch(double (&v)[2]) {
 template <int COLL, typename R>
 __device__ __forceinline__ void batch_collide(R *G, R gx, R gy, R om2, R om3, R om4, bool trim) {
     const R z = R(0);
-    if constexpr (COLL == SMRT_TRIM) collide_smrt_trim<D2Q9>(G, gx, gy, z, om2);
-    else if constexpr (COLL == SMRT) {
-        if (trim) collide_smrt_trim<D2Q9>(G, gx, gy, z, om2);
-        else collide_smrt<D2Q9>(G, gx, gy, z, om2, om3, om4, om2);
-    } else if constexpr (COLL == SMRT_FNEQ) collide_smrt_fneq<D2Q9>(G, gx, gy, z, om2, om3, om4, om2);
-    else if constexpr (COLL == MRT_RAW) collide_mrt_raw<D2Q9>(G, gx, gy, z, om2, om3, om4);
-    else collide_bgk<D2Q9>(G, gx, gy, z, om2);
+    if constexpr (COLL == SMRT) {
+        if (trim) {
+            collide_any<D2Q9, SMRT_TRIM>(G, gx, gy, z, om2, om3, om4, om2);
+            return;
+        }
+    }
+    collide_any<D2Q9, COLL>(G, gx, gy, z, om2, om3, om4, om2);
 }
 
 // One FP32 node of a channel on the pair instructions (both lanes), out of

@@ -6,6 +6,9 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <type_traits>
+
+#include "lbm_collide64.cuh"
 #include "lbm_device.cuh"
 #include "lbm_f32x2.cuh"
 
@@ -14,7 +17,11 @@ namespace lbm {
 // the collision selected by COLL on one node's grid G (or two nodes' with F2)
 template <int L, int COLL, typename R>
 __device__ __forceinline__ void collide_any(R *G, R gx, R gy, R gz, R om2, R om3, R om4, R omb) {
-    if constexpr (COLL == SMRT) collide_smrt<L>(G, gx, gy, gz, om2, om3, om4, omb);
+    // FP64: the forms with fewer FP64 instructions (lbm_collide64.cuh)
+    if constexpr (std::is_same<R, double>::value && COLL == BGK) collide_bgk64<L>(G, gx, gy, gz, om2);
+    else if constexpr (std::is_same<R, double>::value && COLL == SMRT_TRIM && L == D2Q9)
+        collide_smrt_trim64(G, gx, gy, om2);
+    else if constexpr (COLL == SMRT) collide_smrt<L>(G, gx, gy, gz, om2, om3, om4, omb);
     else if constexpr (COLL == SMRT_TRIM) collide_smrt_trim<L>(G, gx, gy, gz, om2);
     else if constexpr (COLL == SMRT_FNEQ) collide_smrt_fneq<L>(G, gx, gy, gz, om2, om3, om4, omb);
     else if constexpr (COLL == MRT_RAW) collide_mrt_raw<L>(G, gx, gy, gz, om2, om3, om4);
