@@ -398,6 +398,7 @@ def run_gpu(args, ws, rank, local):
     total_ms = sum(region_ms)
     kern_ms = sum(es.elapsed_time(ee) for es, ee, _ in chunk_ev) / sum(n for _, _, n in chunk_ev)
     bx, npt, layout = lat.launch()
+    K = lat.launch_steps()   # time steps one kernel launch advances
     u_stall = lat.force_resolution()
     ck = checks[:max(1, k)].cpu().numpy()
     finite = bool(np.all(ck[:, 6] == 0)) and bool(np.all(np.isfinite(ck)))
@@ -408,12 +409,15 @@ def run_gpu(args, ws, rank, local):
     all_steps = steps * repeats
     value = job_rate(ws, N * all_steps, total_ms * 1e-3) / 1e6
     peak, peak_kind = measured_peaks()
+    # one launch reads and writes every population once, for its K steps
     algo_bytes = bytes_per_node * N
-    achieved = algo_bytes / (kern_ms * 1e-3) / 1e9
-    traffic = (traffic_per_launch(N, coll) if st == "F32" and not args.tau_bulk and spec["lattice"] == "D2Q9"
-               else None)
+    achieved = algo_bytes / (kern_ms * K * 1e-3) / 1e9
+    traffic = (traffic_per_launch(N, coll)
+               if st == "F32" and not args.tau_bulk and spec["lattice"] == "D2Q9" and K == 1 else None)
     clocks = sampler.summary()
-    launches = all_steps + 2 * k   # step kernels, and the moments and finalize kernels per check
+    # step kernels (runs of n steps: K per launch, what is left over in smaller ones), and the moments and finalize
+    # kernels per check
+    launches = sum(n // K + (n % K) // 2 + (n % K) % 2 if K > 1 else n for _, _, n in chunk_ev) + 2 * k
 
     e2e = None
     if not args.no_e2e:
@@ -449,11 +453,13 @@ def run_gpu(args, ws, rank, local):
                               "replicas": ws}),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": (f"k_step_vec<{L},{kname},{st},{npt}>" if layout
+                         "kernel": (f"k_step_tile<{kname},{st},{K} steps>" if K > 1 else
+                                    f"k_step_vec<{L},{kname},{st},{npt}>" if layout
                                     else f"k_step<{L},{kname},{st},{npt}>"),
+                         "steps_per_launch": K,
                          "launch": {"block_x": bx, "nodes_per_thread": npt, "layout": "vector" if layout else "strided"},
                          "bytes_per_launch": algo_bytes,
-                         "avg_launch_ms": kern_ms, "peak_source": f"{peak_kind} hbm_gbs (copy)"},
+                         "avg_launch_ms": kern_ms * K, "peak_source": f"{peak_kind} hbm_gbs (copy)"},
             "gpu_launches": launches, "clocks": clocks,
             "check": {"finite": finite, "mass_drift": mass_drift, "residual_K": res},
             "storage_resolution": {"u_stall": u_stall,

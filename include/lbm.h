@@ -211,7 +211,8 @@ lbm_status lbm_set_state(lbm_handle *h, const void *host, size_t bytes, int64_t 
  *     given by lbm_launch_widths. */
 typedef enum { LBM_LAYOUT_STRIDED = 0, LBM_LAYOUT_VECTOR = 1 } lbm_layout;
 
-/* Launch shape of the fused stream-collide kernel: threads per block along x
+/* Launch shape of the fused stream-collide kernel, one step per launch from
+ * then on (see lbm_get_launch_steps): threads per block along x
  * (block_x: 32, 64, 128 or 256), nodes per thread along x and their layout.
  * Drops the captured step graphs;
  * synchronises the handle's stream.  The physics does not depend on the
@@ -227,17 +228,25 @@ lbm_status lbm_set_launch_layout(lbm_handle *h, int block_x, int nodes_per_threa
 lbm_status lbm_set_launch(lbm_handle *h, int block_x, int nodes_per_thread);
 /* The current launch shape (outputs nullable). */
 lbm_status lbm_get_launch(const lbm_handle *h, int *block_x, int *nodes_per_thread, int *layout);
+/* Time steps that one kernel launch of a long lbm_step advances: 2 or 4 on a
+ * new D2Q9 handle in FP32, FP16 or BF16 storage (the steps between kept in
+ * shared memory; bit for bit the result of single steps, to which lbm_step
+ * falls back for what is left over), else 1.  lbm_set_launch and
+ * lbm_set_launch_layout set 1; lbm_autotune keeps what it measures faster. */
+lbm_status lbm_get_launch_steps(const lbm_handle *h, int *steps);
 /* The two vector widths (nodes per thread; equal when only one is built) of
  * LBM_LAYOUT_VECTOR for a lattice and storage (outputs nullable). */
 lbm_status lbm_launch_widths(int lattice, int storage, int *lo, int *hi);
 
-/* Time every supported launch shape over `trials` launches each (CUDA events
+/* Time several steps per launch (where lbm_get_launch_steps gives more than 1
+ * on a new handle) and every supported launch shape over `trials` launches each (CUDA events
  * on the handle's stream; the kernel reads the current state and writes the
  * spare buffer, so the state does not advance): the strided shapes, and the
  * vector shapes (blocks of 32, 64, 128; both widths) where
  * that layout applies.  Keep the fastest and return its block_x and
- * nodes_per_thread (outputs nullable; lbm_get_launch gives its layout) with
- * its mean launch time in milliseconds.  Synchronises. */
+ * nodes_per_thread (outputs nullable; lbm_get_launch gives its layout; with
+ * several steps per launch, the shape left for single steps) with its mean
+ * time per step in milliseconds.  Synchronises. */
 lbm_status lbm_autotune(lbm_handle *h, int trials, int *block_x, int *nodes_per_thread, double *ms);
 
 /* Information (outputs nullable): D, Q, the step counter, and the

@@ -83,6 +83,7 @@ def library():
     L.lbm_set_launch.argtypes = [H, C.c_int, C.c_int]
     L.lbm_set_launch_layout.argtypes = [H, C.c_int, C.c_int, C.c_int]
     L.lbm_get_launch.argtypes = [H, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int)]
+    L.lbm_get_launch_steps.argtypes = [H, C.POINTER(C.c_int)]
     L.lbm_launch_widths.argtypes = [C.c_int, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_int)]
     L.lbm_force_resolution.argtypes = [H, dp]
     L.lbm_alu_peak.argtypes = [C.c_int, C.c_int64, dp, dp]
@@ -129,6 +130,7 @@ def library():
               "lbm_check_device",
               "lbm_set_force", "lbm_set_force_schedule", "lbm_set_force_scale_schedule", "lbm_get_populations", "lbm_set_populations", "lbm_get_state",
               "lbm_set_state", "lbm_info", "lbm_set_launch", "lbm_set_launch_layout", "lbm_get_launch",
+              "lbm_get_launch_steps",
               "lbm_launch_widths", "lbm_force_resolution", "lbm_alu_peak", "lbm_autotune", "lbm_check_noalloc", "lbm_split_schedule", "lbm_split_create",
               "lbm_split_step", "lbm_split_check_device", "lbm_split_moments", "lbm_split_get_state",
               "lbm_split_get_populations", "lbm_split_set_launch_layout",
@@ -302,6 +304,12 @@ def lbm_get_launch(h):
     return bx.value, npt.value, lay.value
 
 
+def lbm_get_launch_steps(h):
+    k = C.c_int()
+    _check(library().lbm_get_launch_steps(h, C.byref(k)), h)
+    return k.value
+
+
 def lbm_launch_widths(lattice, storage):
     lo, hi = C.c_int(), C.c_int()
     _check(library().lbm_launch_widths(_enum("lattice", lattice), _enum("storage", storage), C.byref(lo),
@@ -448,6 +456,10 @@ class Lattice:
         """(block_x, nodes_per_thread, layout) of the step kernel."""
         return lbm_get_launch(self.h)
 
+    def launch_steps(self):
+        """Time steps per kernel launch of a long step() (see lbm_get_launch_steps)."""
+        return lbm_get_launch_steps(self.h)
+
     def force_resolution(self):
         """Speed above which one step of the force rounds away in the storage
         format (see lbm_force_resolution); inf without a force."""
@@ -467,7 +479,10 @@ class Lattice:
             key = A.signature(self)
             hit = A.lookup(cache, key)
             if hit:
-                self.set_launch(*hit["launch"])
+                # the shape a new handle starts with stays as it is: setting
+                # it would give up several steps per launch
+                if tuple(hit["launch"]) != self.launch():
+                    self.set_launch(*hit["launch"])
                 return tuple(hit["launch"]) + (hit["ms"],)
         bx, npt, ms = lbm_autotune(self.h, trials)
         if cache:

@@ -41,7 +41,7 @@ struct BatchChan {
     long long plane;     // nxp * ny
     long long snap_off;  // offset (elements of the arithmetic type) of its velocity snapshot, 2 * nx * ny
     long long part_off;  // offset (doubles) of its tile partials, 2 per tile, room for ny tiles
-    long long solid_off; // offset of its obstacle mask (nxp * ny bytes) in the mask arena, -1: none
+    long long solid_off; // offset of its obstacle mask and links (nxp * ny entries) in their arenas, -1: none
     int nx, ny, nxp;
     int per_x, per_y;
     double om2, om3, om4;
@@ -73,7 +73,7 @@ struct BatchRun {
     const BatchChan *ch;
     BatchCtl *ctl;
     int n;
-    const unsigned char *solid;  // mask arena
+    const unsigned *links;       // obstacle links of the channels with a mask
     int grid;                  // resident CTAs
     int tile_min, tile_max;    // nodes per tile
     long long *active_nodes;   // nodes of channels still running
@@ -103,12 +103,13 @@ __device__ __forceinline__ T vload(const T *p) { return *(const volatile T *)p; 
 // base, all offsets within a channel fit in 32 bits
 template <int ST>
 __device__ __forceinline__ void gather_chan(const BatchChan &C, const typename Store<ST>::T *f,
-                                            const unsigned char *solid, int x, int y,
+                                            const unsigned *links, int x, int y,
                                             typename Store<ST>::R *G) {
     typedef typename Store<ST>::R R;
     typedef typename Store<ST>::T T;
     const int plane = (int)C.plane;
     const int own = y * C.nxp + x;
+    const unsigned link = links ? links[own] : 0u;
     // no wall or wrap along y, and x inside the row or periodic (the row's
     // first and last nodes then take their x - c_x across the periodic face)
     const bool interior = ((x > 0 && x < C.nx - 1) || C.per_x) && y > 0 && y < C.ny - 1;
@@ -128,7 +129,7 @@ __device__ __forceinline__ void gather_chan(const BatchChan &C, const typename S
             else if (sy >= C.ny) { if (C.per_y) sy -= C.ny; else wall = true; }
             src = sy * C.nxp + sx;
         }
-        if (solid && i != 0 && !wall) wall = solid[src] != 0;
+        if (i != 0) wall = wall || ((link >> i) & 1u);
         const int idx = wall ? opp<D2Q9>(i) * plane + own : i * plane + src;
         G[gpos<D2Q9>(i)] = (R)ld_cg<T>(f + idx);
     }
@@ -178,10 +179,10 @@ __device__ __forceinline__ void batch_collide(R *G, R gx, R gy, R om2, R om3, R 
 // kernel keeps one inlined pair collision per collision kind
 template <int COLL>
 __device__ __noinline__ void batch_node_alone(const BatchChan C, const float *fin, float *fout,
-                                              const unsigned char *solid, int x, int y, float gx, float gy,
+                                              const unsigned *links, int x, int y, float gx, float gy,
                                               float om2, float om3, float om4, bool trim) {
     float G[9];
-    gather_chan<ST_F32>(C, fin, solid, x, y, G);
+    gather_chan<ST_F32>(C, fin, links, x, y, G);
     F2 G2[9];
 #pragma unroll
     for (int g = 0; g < 9; ++g) G2[g] = F2(G[g]);
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(256, 4) k_batch(const BatchRun r) {
             const int y1 = min(y0 + rows, C.ny);
             const int nn = y1 > y0 ? (y1 - y0) * C.nx : 0;  // the last tiles may be empty
             R *snap = (R *)r.snap + C.snap_off;
-            const unsigned char *solid = C.solid_off >= 0 ? r.solid + C.solid_off : nullptr;
+            const unsigned *links = C.solid_off >= 0 ? r.links + C.solid_off : nullptr;
             const int N = C.nx * C.ny;
             const R om2 = R(C.om2), om3 = R(C.om3), om4 = R(C.om4), gx = R(C.gx), gy = R(C.gy);
             const bool trim = C.om3 == 1.0 && C.om4 == 1.0;
@@ -325,8 +326,8 @@ __global__ void __launch_bounds__(256, 4) k_batch(const BatchRun r) {
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     on[k] = base + k * (int)blockDim.x < nn;
-                    if (on[k] && solid) on[k] = solid[ys[k] * C.nxp + xs[k]] == 0;
-                    if (on[k]) gather_chan<ST>(C, fin, solid, xs[k], ys[k], G[k]);
+                    if (on[k] && links) on[k] = (links[ys[k] * C.nxp + xs[k]] & 1u) == 0u;
+                    if (on[k]) gather_chan<ST>(C, fin, links, xs[k], ys[k], G[k]);
                 }
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
@@ -367,8 +368,8 @@ __global__ void __launch_bounds__(256, 4) k_batch(const BatchRun r) {
                         }
                     } else {
                         // a node alone (the tile's last pass): out of line
-                        if (on[0]) batch_node_alone<COLL>(C, fin, fout, solid, xs[0], ys[0], gx, gy, om2, om3, om4, trim);
-                        if (on[1]) batch_node_alone<COLL>(C, fin, fout, solid, xs[1], ys[1], gx, gy, om2, om3, om4, trim);
+                        if (on[0]) batch_node_alone<COLL>(C, fin, fout, links, xs[0], ys[0], gx, gy, om2, om3, om4, trim);
+                        if (on[1]) batch_node_alone<COLL>(C, fin, fout, links, xs[1], ys[1], gx, gy, om2, om3, om4, trim);
                     }
                 } else {
 #pragma unroll
@@ -497,6 +498,7 @@ struct lbm_batch {
     float *g32_dev = nullptr;   // per channel 4 floats
     double *fields = nullptr;   // initial rho0 / u0, per channel, when given
     unsigned char *solid = nullptr;  // obstacle masks of the channels that have one
+    unsigned *links = nullptr;       // their obstacle links (KParams.links), at the same offsets
     std::vector<long long> field_off;
     BatchChan *ch_dev = nullptr;
     BatchCtl *ctl_dev = nullptr;
@@ -601,7 +603,7 @@ lbm_status batch_run(lbm_batch *b, double tol, int K, int64_t max_steps) {
     r.ch = b->ch_dev;
     r.ctl = b->ctl_dev;
     r.n = b->n;
-    r.solid = b->solid;
+    r.links = b->links;
     // at most 4000 CTAs: the tile field of the claim word overshoots the tile
     // count (<= 4096) by at most the number of concurrent claimers (< 8192 - 4096)
     r.grid = std::min(sms * per_sm, 4000);
@@ -842,7 +844,7 @@ void lbm_batch_destroy(lbm_batch *b) {
     if (b->stream) cudaStreamSynchronize(b->stream);
     void *ptrs[] = {b->fa,      b->fb,       b->snap,         b->part,  b->g_dev,    b->g32_dev,
                     b->fields,  b->ch_dev,   b->ctl_dev,      b->active_count, b->error, b->progress,
-                    b->active_nodes, b->active_bits, b->partials, b->red, b->tmp, b->solid};
+                    b->active_nodes, b->active_bits, b->partials, b->red, b->tmp, b->solid, b->links};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
@@ -948,7 +950,8 @@ lbm_status lbm_batch_create(const lbm_desc *descs, int n, lbm_batch **out) {
         (st = balloc(b, &b->active_bits, (size_t)((n + 31) / 32) * 4)) ||
         (st = balloc(b, &b->partials, (size_t)kMomGridMax * kPartials * 8)) || (st = balloc(b, &b->red, 64)) ||
         (fields && (st = balloc(b, &b->fields, (size_t)fields * 8))) ||
-        (solid_bytes && (st = balloc(b, &b->solid, (size_t)solid_bytes)))) {
+        (solid_bytes && ((st = balloc(b, &b->solid, (size_t)solid_bytes)) ||
+                         (st = balloc(b, &b->links, (size_t)solid_bytes * sizeof(unsigned)))))) {
         std::string m = b->err;
         lbm_batch_destroy(b);
         return bfail(nullptr, st, m);
@@ -974,6 +977,7 @@ lbm_status lbm_batch_create(const lbm_desc *descs, int n, lbm_batch **out) {
         k.per[2] = 1;
         k.force_kind = d.force_kind == LBM_G_UNIFORM ? G_UNIFORM : G_NONE;
         k.solid = d.solid ? b->solid + b->ch[c].solid_off : nullptr;
+        k.links = d.solid ? b->links + b->ch[c].solid_off : nullptr;
         k.g = b->g_dev + 4 * c;
         k.g32 = b->g32_dev + 4 * c;
         for (int m = 0; m < 5; ++m) {
@@ -992,6 +996,10 @@ lbm_status lbm_batch_create(const lbm_desc *descs, int n, lbm_batch **out) {
         e = cudaMemcpyAsync(b->solid + b->ch[c].solid_off, m.data(), m.size(), cudaMemcpyHostToDevice, b->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     }
+    if (e == cudaSuccess && solid_bytes)
+        e = cudaMemsetAsync(b->links, 0, (size_t)solid_bytes * sizeof(unsigned), b->stream);
+    for (int c = 0; c < n && e == cudaSuccess; ++c)
+        if (descs[c].solid) e = launchers_d2q9().links(b->kp[c], b->links + b->ch[c].solid_off, nullptr, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->g32_dev, g32.data(), g32.size() * 4, cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->fa, 0, (size_t)off * eb, b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->fb, 0, (size_t)off * eb, b->stream);

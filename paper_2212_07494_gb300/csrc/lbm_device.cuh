@@ -167,6 +167,11 @@ struct KParams {
     const double *g;               // uniform [3] | rows [ny][D] | field [D][plane]
     const float *g32;              // the same force in FP32 (for FP32 arithmetic)
     const unsigned char *solid;    // [plane] or null
+    // obstacle links [plane], made from the mask once (with it or null): bit
+    // i, population i of the node is pulled from a solid node, i.e. bounces
+    // back; bit 0, the node itself is solid.  One load per node instead of
+    // one mask byte per population.
+    const unsigned *links;
     double om[5];                  // 1 / tau_n
     float om32[5];
     double omb;                    // 1 / tau of the trace (bulk) part of order 2; om[2] unless split
@@ -184,17 +189,15 @@ struct KParams {
     // (the node itself, or its neighbour along x, wrapped on a periodic x):
     long long doff[27];            // i*plane - (cy*nxp + cz*nxp*ny): pull source
     long long poff[27];            // i*plane: the node's own entry (relative to the node)
-    int noff[27];                  // -(cy*nxp + cz*nxp*ny): neighbour x - c_i
 };
 
 // fill the per-population offsets of KParams for lattice L (host side)
 template <int L> inline void fill_offsets(KParams &p) {
-    for (int i = 0; i < 27; ++i) p.doff[i] = p.poff[i] = p.noff[i] = 0;
+    for (int i = 0; i < 27; ++i) p.doff[i] = p.poff[i] = 0;
     for (int i = 0; i < Lat<L>::Q; ++i) {
         const long long nb = (long long)Lat<L>::cy(i) * p.nxp + (long long)Lat<L>::cz(i) * p.nxp * p.ny;
         p.poff[i] = (long long)i * p.plane;
         p.doff[i] = p.poff[i] - nb;
-        p.noff[i] = (int)(-nb);
     }
 }
 
@@ -265,6 +268,9 @@ template <int L, typename R> __host__ __device__ __forceinline__ void reconstruc
     }
 }
 
+// 1 / rho; the pair type has an overload of its own (lbm_f32x2.cuh)
+template <typename R> __host__ __device__ __forceinline__ R one_over(R rho) { return R(1) / rho; }
+
 // ------------------------------------------------------------------ collisions
 // Second-order central moments scaled by (1 - a) in their traceless (shear)
 // part and (1 - b) in their trace (bulk) part, Eq. (domg) with tau_{2,2} and
@@ -295,7 +301,7 @@ __host__ __device__ __forceinline__ void collide_smrt(R *G, R gx, R gy, R gz, R 
     project<D>(G);
     const R drho = G[0];                 // rho - 1 (moments of w vanish beyond order 0)
     const R rho = R(1) + drho;
-    const R inv = R(1) / rho;
+    const R inv = one_over(rho);
     const R ux = G[EX] * inv + R(0.5) * gx;   // Eq. (half_F)
     const R uy = G[EY] * inv + R(0.5) * gy;
     const R uz = D == 3 ? G[EZ] * inv + R(0.5) * gz : R(0);
@@ -462,7 +468,7 @@ __host__ __device__ __forceinline__ void collide_smrt_trim(R *G, R gx, R gy, R g
     if constexpr (D == 3) proj_pass<D, 2, P3>(G);
     const R drho = G[0];
     const R rho = R(1) + drho;
-    const R inv = R(1) / rho;
+    const R inv = one_over(rho);
     const R ux = G[EX] * inv + R(0.5) * gx;   // Eq. (half_F)
     const R uy = G[EY] * inv + R(0.5) * gy;
     const R uz = D == 3 ? G[EZ] * inv + R(0.5) * gz : R(0);
@@ -519,7 +525,7 @@ __host__ __device__ __forceinline__ void collide_smrt_fneq(R *G, R gx, R gy, R g
     project<D>(G);
     const R drho = G[0];
     const R rho = R(1) + drho;
-    const R inv = R(1) / rho;
+    const R inv = one_over(rho);
     const R ux = G[EX] * inv + R(0.5) * gx;   // Eq. (half_F)
     const R uy = G[EY] * inv + R(0.5) * gy;
     const R uz = D == 3 ? G[EZ] * inv + R(0.5) * gz : R(0);
@@ -586,7 +592,7 @@ __host__ __device__ __forceinline__ void collide_mrt_raw(R *G, R gx, R gy, R gz,
     project<D>(G);
     const R drho = G[0];
     const R rho = R(1) + drho;
-    const R inv = R(1) / rho;
+    const R inv = one_over(rho);
     const R ux = G[EX] * inv + R(0.5) * gx;   // Eq. (half_F)
     const R uy = G[EY] * inv + R(0.5) * gy;
     const R uz = D == 3 ? G[EZ] * inv + R(0.5) * gz : R(0);
@@ -648,7 +654,7 @@ __host__ __device__ __forceinline__ void collide_bgk(R *G, R gx, R gy, R gz, R o
         if (D == 3 && Lat<L>::cz(i)) jz += Lat<L>::cz(i) > 0 ? v : -v;
     }
     const R rho = R(1) + drho;
-    const R inv = R(1) / rho;
+    const R inv = one_over(rho);
     const R ux = jx * inv + R(0.5) * gx, uy = jy * inv + R(0.5) * gy;
     const R uz = D == 3 ? jz * inv + R(0.5) * gz : R(0);
     const R uu15 = R(1.5) * (ux * ux + uy * uy + uz * uz);
@@ -781,6 +787,7 @@ __device__ __forceinline__ void gather(const KParams &p, const typename Store<ST
     // x face, so the first and last nodes of a row take this path too
     const bool interior = ((x > 0 && x < p.nx - 1) || p.per[0]) && inner(p, 1, y, p.ny) &&
                           (D == 2 || inner(p, 2, z, p.nz));
+    const unsigned link = MASK ? __ldg(p.links + own) : 0u;
     if (interior) {
         const long long xl = x == 0 ? p.nx - 1 : -1;          // to x - 1
         const long long xr = x == p.nx - 1 ? 1 - p.nx : 1;    // to x + 1
@@ -788,9 +795,8 @@ __device__ __forceinline__ void gather(const KParams &p, const typename Store<ST
 #pragma unroll
         for (int i = 0; i < Lat<L>::Q; ++i) {
             const int cx = Lat<L>::cx(i);
-            const long long sx = cx == 1 ? xl : (cx == -1 ? xr : 0);
             const typename Store<ST>::T *src = cx == 1 ? basel : (cx == -1 ? baser : base);
-            if (MASK && i != 0 && p.solid[own + sx + p.noff[i]] != 0)
+            if (MASK && i != 0 && ((link >> i) & 1u))
                 G[gpos<L>(i)] = Store<ST>::ld(base + p.poff[opp<L>(i)]);
             else
                 G[gpos<L>(i)] = Store<ST>::ld(src + p.doff[i]);
@@ -804,7 +810,7 @@ __device__ __forceinline__ void gather(const KParams &p, const typename Store<ST
         const int kx = Lat<L>::cx(i) + 1, ky = Lat<L>::cy(i) + 1, kz = Lat<L>::cz(i) + 1;
         bool wall = nb.xw[kx] || nb.yw[ky] || (D == 3 && nb.zw[kz]);
         const long long src = node_index(p, nb.xs[kx], nb.ys[ky], D == 3 ? nb.zs[kz] : z);
-        if (MASK && i != 0 && !wall) wall = p.solid[src] != 0;
+        if (MASK && i != 0) wall = wall || ((link >> i) & 1u);
         const long long idx = wall ? p.poff[opp<L>(i)] + own : p.poff[i] + src;
         G[gpos<L>(i)] = Store<ST>::ld(f + idx);
     }

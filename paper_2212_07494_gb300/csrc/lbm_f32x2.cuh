@@ -108,4 +108,13 @@ __device__ __forceinline__ float f1_div(float a, float b) {
 // a / b per lane, each correctly rounded
 __device__ __forceinline__ F2 operator/(F2 a, F2 b) { return F2::pair(f1_div(a.lo(), b.lo()), f1_div(a.hi(), b.hi())); }
 
+// 1 / b per lane, correctly rounded (rcp.rn.f32): the bits of the quotient
+// 1 / b, in fewer instructions than the general division
+__device__ __forceinline__ F2 one_over(F2 b) {
+    float lo, hi;
+    asm("rcp.rn.f32 %0, %1;" : "=f"(lo) : "f"(b.lo()));
+    asm("rcp.rn.f32 %0, %1;" : "=f"(hi) : "f"(b.hi()));
+    return F2::pair(lo, hi);
+}
+
 }  // namespace lbm

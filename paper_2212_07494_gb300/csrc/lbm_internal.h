@@ -97,6 +97,37 @@ inline StepVecFn step_vec_fn(int lattice, int storage) {
     return t[lattice][storage];
 }
 
+// what k_step_tile needs to know of its domain (a lattice, or a channel of a
+// batch)
+struct TileDom {
+    int nx, ny, nxp, per_x, per_y;
+    unsigned plane_bytes;           // bytes of one population plane (< 2^32)
+    const unsigned *links;          // obstacle links (KParams.links), or null without a mask
+    int force_kind;
+    const float *g;                 // force of the first step (load_force layout); step s reads g + s * g_step
+    long long g_step, g_plane;      // values between the forces of successive steps; of a per-node force's components
+    float om2, om3, om4, omb;
+    bool trim;                      // SMRT with tau_3 = tau_4 = 1 and one second-order tau: the trimmed collision
+};
+
+// k_step_tile launcher of one storage type, K = 2 or 4 steps (cudaErrorInvalidValue otherwise)
+typedef cudaError_t (*StepTileFn)(int coll, int K, const TileDom &d, const void *fin, void *fout, cudaStream_t s);
+cudaError_t step_tile_f32(int, int, const TileDom &, const void *, void *, cudaStream_t);
+cudaError_t step_tile_f16(int, int, const TileDom &, const void *, void *, cudaStream_t);
+cudaError_t step_tile_bf16(int, int, const TileDom &, const void *, void *, cudaStream_t);
+cudaError_t step_tile_mask_f32(int, int, const TileDom &, const void *, void *, cudaStream_t);
+cudaError_t step_tile_mask_f16(int, int, const TileDom &, const void *, void *, cudaStream_t);
+cudaError_t step_tile_mask_bf16(int, int, const TileDom &, const void *, void *, cudaStream_t);
+
+inline StepTileFn step_tile_fn(int storage, bool mask) {
+    switch (storage) {
+    case ST_F32: return mask ? step_tile_mask_f32 : step_tile_f32;
+    case ST_F16: return mask ? step_tile_mask_f16 : step_tile_f16;
+    case ST_BF16: return mask ? step_tile_mask_bf16 : step_tile_bf16;
+    }
+    return nullptr;
+}
+
 struct Launchers {
     cudaError_t (*step)(int coll, int st, bool mask, StepCfg cfg, const KParams &p, const void *fin,
                         void *fout, cudaStream_t s);
@@ -112,6 +143,8 @@ struct Launchers {
     cudaError_t (*get_pops)(int st, bool mask, const KParams &p, const void *state, double *out,
                             cudaStream_t s);
     cudaError_t (*put_pops)(int st, const KParams &p, const double *in, void *target, cudaStream_t s);
+    // obstacle links of every node from p.solid (KParams.links); *linked (device, may be null) += nodes with any
+    cudaError_t (*links)(const KParams &p, unsigned *links, unsigned *linked, cudaStream_t s);
 };
 
 const Launchers &launchers_d2q9();

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256, step_min_blocks<ST>()) k_step(const __gri
     for (int k = 0; k < NPT; ++k) {
         const int x = x0 + k * blockDim.x;
         act[k] = x < p.nx;
-        if (MASK && act[k]) act[k] = p.solid[node_index(p, x, y, z)] == 0;
+        if (MASK && act[k]) act[k] = (__ldg(p.links + node_index(p, x, y, z)) & 1u) == 0u;
         if (act[k]) gather<L, ST, MASK>(p, fin, x, y, z, G[k]);
     }
     const R om2 = omega<R>(p, 2), om3 = omega<R>(p, 3), om4 = omega<R>(p, 4), omb = omega_bulk<R>(p);
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kMomBlock) k_moments(const KParams p, const ty
         for (int k = 0; k < kMomNpt; ++k) {
             const int x = seg * SEG + k * kMomBlock + threadIdx.x;
             on[k] = x < p.nx;
-            fl[k] = on[k] && (!MASK || p.solid[node_index(p, x, y, z)] == 0);
+            fl[k] = on[k] && (!MASK || (__ldg(p.links + node_index(p, x, y, z)) & 1u) == 0u);
             if (fl[k]) gather<L, ST, MASK>(p, f, x, y, z, G[k]);
         }
         // the snapshot is read for all nodes of the work item before any of
@@ -330,6 +330,31 @@ __global__ void k_unstream(const KParams p, const typename Store<ST>::T *__restr
         const long long idx = wall ? (long long)opp<L>(j) * p.plane + own : (long long)j * p.plane + dst;
         P[(long long)j * p.plane + own] = T[idx];
     }
+}
+
+// Obstacle links of every node a pull can be asked for (a slab's halo layers
+// excluded) from the mask.  linked: number of nodes with any link or solid.
+template <int L>
+__global__ void k_links(const KParams p, unsigned *__restrict__ links, unsigned *linked) {
+    const int y = blockIdx.y + (p.halo_ax == 1), z = blockIdx.z + (p.halo_ax == 2);
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned b = 0u;
+    if (x < p.nx) {
+        const long long own = node_index(p, x, y, z);
+        NodeNbr nb;
+        node_nbr(p, x, y, z, nb);
+        b = p.solid[own] ? 1u : 0u;
+#pragma unroll
+        for (int i = 1; i < Lat<L>::Q; ++i) {
+            const int kx = Lat<L>::cx(i) + 1, ky = Lat<L>::cy(i) + 1, kz = Lat<L>::cz(i) + 1;
+            const bool wall = nb.xw[kx] || nb.yw[ky] || (Lat<L>::D == 3 && nb.zw[kz]);
+            const long long src = node_index(p, nb.xs[kx], nb.ys[ky], Lat<L>::D == 3 ? nb.zs[kz] : z);
+            if (!wall && p.solid[src] != 0) b |= 1u << i;
+        }
+        links[own] = b;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, b != 0u);
+    if (linked && m != 0u && (threadIdx.x & 31) == 0) atomicAdd(linked, (unsigned)__popc(m));
 }
 
 // Pre-collision populations fbar = w + delta in FP64, unpadded [Q][N]
@@ -500,8 +525,13 @@ template <int L> struct Dispatch {
         return cudaErrorInvalidValue;
     }
 
+    static cudaError_t links(const KParams &p, unsigned *out, unsigned *linked, cudaStream_t s) {
+        k_links<L><<<step_grid(p, 128, 1), 128, 0, s>>>(p, out, linked);
+        return cudaGetLastError();
+    }
+
     static const Launchers &table() {
-        static const Launchers t = {&step, &moments, &init, &unstream, &get_pops, &put_pops};
+        static const Launchers t = {&step, &moments, &init, &unstream, &get_pops, &put_pops, &links};
         return t;
     }
 };

@@ -92,6 +92,25 @@ __global__ void k_sched_apply(const double *table, const long long *t, int off, 
     }
 }
 
+// The forces of the next n steps of a schedule at once: ring[i * count ..] =
+// entry *t + i for i < n, and entry *t + n, the force after them, into the
+// force buffers g / g32.  With one value per step and a table of uniform
+// forces (scale = 0) count is 3.
+__global__ void k_sched_fill(const double *table, const long long *t, int n, int scale, const double *base,
+                             long long count, double *ring, float *ring32, double *g, float *g32) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (n + 1) * count) return;
+    const long long s = i / count, j = i - s * count;
+    const double v = scale ? table[*t + s] * base[j] : table[3 * (*t + s) + j];
+    if (s < n) {
+        ring[i] = v;
+        ring32[i] = (float)v;
+    } else {
+        g[j] = v;
+        g32[j] = (float)v;
+    }
+}
+
 cudaError_t launch_finalize(const double *partials, int nblocks, double *out, cudaStream_t s) {
     k_finalize<<<1, 256, 0, s>>>(partials, nblocks, out);
     return cudaGetLastError();
@@ -114,6 +133,7 @@ struct lbm_handle {
     double *g_dev = nullptr;
     size_t g_count = 0;       // doubles in the host layout of g
     unsigned char *solid_dev = nullptr;
+    unsigned *links_dev = nullptr;   // obstacle links of the mask (KParams.links)
     double *partials = nullptr;
     int max_blocks = 0;
     double *red_dev = nullptr;   // 8 doubles: M, Px, Py, Pz, res num, res den, non-finite
@@ -132,7 +152,14 @@ struct lbm_handle {
     bool gs_scale = false;       // gs_dev holds a scale schedule
     long long *gs_t_dev = nullptr;
     int64_t gs_period = 0;
+    // forces of the next 64 steps under a schedule (null when 64 copies of
+    // the force are too many: then each step's force is written after the
+    // step before it)
+    double *gring_dev = nullptr;
+    float *gring32_dev = nullptr;
     int graph_steps = 0;
+    bool fuse = false;           // several steps per launch (k_step_tile)
+    bool hold_fuse = false;      // not in the current call (a caller's stream capture)
     int64_t step = 0;
     void *(*alloc)(size_t, void *) = nullptr;
     void (*free_)(void *, void *) = nullptr;
@@ -254,26 +281,99 @@ bool shape_ok(const lbm_handle *h, StepCfg c) {
     return c.npt == vec_width_lo(h->lattice, h->storage) || c.npt == vec_width_hi(h->lattice, h->storage);
 }
 
-lbm_status launch_steps(lbm_handle *h, int64_t n) {
-    int since = 0;   // with a force schedule: steps since the counter last advanced (< 64)
-    for (int64_t s = 0; s < n; ++s) {
-        cudaError_t e = launch_step(h, h->cfg, h->buf[h->cur], h->buf[1 - h->cur]);
-        if (e != cudaSuccess) return cuda_fail(h, e, "stream-collide launch");
+// k_step_tile takes 32-bit byte offsets into a whole D2Q9 domain (not a slab)
+// at least as wide as its margins, in FP32 arithmetic
+bool tile_ok(const lbm_handle *h) {
+    return h->lattice == LBM_D2Q9 && h->storage != LBM_F64 && h->kp.halo_ax == 0 && h->nx > 4 && h->ny > 4 &&
+           (long long)h->Q * h->kp.plane * (long long)storage_bytes(h->storage) < (1LL << 32);
+}
+
+// Steps of one launch when `left` are wanted.  Small domains take four per
+// launch: a launch's latency (about 2.3 us for two steps) bounds them, and
+// the margins' extra collisions are hidden.  From about 1.5e5 nodes on the
+// collisions fill the chip and two steps are faster (F32, us per step, four
+// against two: 400 x 300 1.82 / 1.95, 512^2 2.95 / 2.82, 1024^2 9.3 / 7.4).
+int fused_steps(const lbm_handle *h, int64_t left) {
+    if (!h->fuse || h->hold_fuse || !tile_ok(h) || (h->gs_dev && !h->gring_dev)) return 1;
+    if (left >= 4 && (long long)h->nx * h->ny <= 150000) return 4;
+    return left >= 2 ? 2 : 1;
+}
+
+// K steps from fin to fout; g32 and g_step: the first step's force and the
+// distance to the next one's (0: the same)
+cudaError_t launch_tile(lbm_handle *h, int K, const float *g32, long long g_step, const void *fin, void *fout) {
+    const KParams &p = h->kp;
+    TileDom d{};
+    d.nx = p.nx;
+    d.ny = p.ny;
+    d.nxp = p.nxp;
+    d.per_x = p.per[0];
+    d.per_y = p.per[1];
+    d.plane_bytes = (unsigned)(p.plane * (long long)storage_bytes(h->storage));
+    d.links = p.links;
+    d.force_kind = p.force_kind;
+    d.g = g32;
+    d.g_step = g_step;
+    d.g_plane = p.plane;
+    d.om2 = p.om32[2];
+    d.om3 = p.om32[3];
+    d.om4 = p.om32[4];
+    d.omb = p.omb32;
+    d.trim = p.om[3] == 1.0 && p.om[4] == 1.0 && p.omb == p.om[2];
+    return step_tile_fn(h->storage, h->mask)(h->collision, K, d, fin, fout, h->stream);
+}
+
+// n <= 64 steps whose forces lie g_step values apart from g / g32 on (0: one
+// force for all)
+lbm_status launch_run(lbm_handle *h, int n, double *g, float *g32, long long g_step) {
+    KParams &p = h->kp;
+    double *const g0 = const_cast<double *>(p.g);
+    float *const g320 = const_cast<float *>(p.g32);
+    cudaError_t e = cudaSuccess;
+    for (int s = 0; s < n && e == cudaSuccess;) {
+        const int k = fused_steps(h, n - s);
+        const void *fin = h->buf[h->cur];
+        void *fout = h->buf[1 - h->cur];
+        if (k > 1) {
+            e = launch_tile(h, k, g32 + s * g_step, g_step, fin, fout);
+        } else {
+            p.g = g + s * g_step;
+            p.g32 = g32 + s * g_step;
+            e = launch_step(h, h->cfg, fin, fout);
+            p.g = g0;
+            p.g32 = g320;
+        }
         h->cur = 1 - h->cur;
-        if (h->gs_dev) {
-            // the force of the next step
-            lbm_status st = sched_apply(h, since + 1);
-            if (st != LBM_OK) return st;
-        }
-        if (h->gs_dev && ++since == 64) {
-            k_sched_advance<<<1, 1, 0, h->stream>>>(h->gs_t_dev, 64LL, (long long)h->gs_period);
-            LBM_CUDA(h, cudaGetLastError());
-            since = 0;
-        }
+        s += k;
     }
-    if (h->gs_dev && since > 0) {
-        k_sched_advance<<<1, 1, 0, h->stream>>>(h->gs_t_dev, (long long)since, (long long)h->gs_period);
-        LBM_CUDA(h, cudaGetLastError());
+    return e == cudaSuccess ? LBM_OK : cuda_fail(h, e, "stream-collide launch");
+}
+
+lbm_status launch_steps(lbm_handle *h, int64_t n) {
+    while (n > 0) {
+        const int m = (int)std::min<int64_t>(n, 64);
+        n -= m;
+        lbm_status st = LBM_OK;
+        if (h->gs_dev && h->gring_dev) {
+            const long long count = h->gs_scale ? (long long)h->gdev_count : 3;
+            k_sched_fill<<<(unsigned)(((m + 1) * count + 255) / 256), 256, 0, h->stream>>>(
+                h->gs_dev, h->gs_t_dev, m, h->gs_scale ? 1 : 0, h->gbase_dev, count, h->gring_dev, h->gring32_dev,
+                h->g_dev, h->g32_dev);
+            LBM_CUDA(h, cudaGetLastError());
+            st = launch_run(h, m, h->gring_dev, h->gring32_dev, count);
+        } else if (h->gs_dev) {
+            for (int s = 0; s < m && st == LBM_OK; ++s) {
+                st = launch_run(h, 1, h->g_dev, h->g32_dev, 0);
+                if (st == LBM_OK) st = sched_apply(h, s + 1);   // the force of the next step
+            }
+        } else {
+            st = launch_run(h, m, h->g_dev, h->g32_dev, 0);
+        }
+        if (st != LBM_OK) return st;
+        if (h->gs_dev) {
+            k_sched_advance<<<1, 1, 0, h->stream>>>(h->gs_t_dev, (long long)m, (long long)h->gs_period);
+            LBM_CUDA(h, cudaGetLastError());
+        }
     }
     return LBM_OK;
 }
@@ -310,9 +410,13 @@ void free_schedule(lbm_handle *h) {
     dev_free(h, h->gs_dev);
     dev_free(h, h->gbase_dev);
     dev_free(h, h->gs_t_dev);
+    dev_free(h, h->gring_dev);
+    dev_free(h, h->gring32_dev);
     h->gs_dev = nullptr;
     h->gbase_dev = nullptr;
     h->gs_t_dev = nullptr;
+    h->gring_dev = nullptr;
+    h->gring32_dev = nullptr;
     h->gs_period = 0;
     h->gs_scale = false;
 }
@@ -328,7 +432,7 @@ lbm_status ensure_graph(lbm_handle *h) {
     LBM_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
     lbm_status st = launch_steps(h, steps);
     cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-    h->cur = saved;  // capture does not execute; steps is even anyway
+    h->cur = saved;  // capture does not execute, and its launches are even in number
     if (st != LBM_OK) {
         if (g) cudaGraphDestroy(g);
         return st;
@@ -376,6 +480,13 @@ lbm_status set_schedule(lbm_handle *h, const std::vector<double> &table, int64_t
     lbm_status st = alloc_into(h, &h->gs_dev, tmp.size() * sizeof(double), "force schedule");
     if (st == LBM_OK) st = alloc_into(h, &h->gs_t_dev, sizeof(long long), "force schedule counter");
     if (st == LBM_OK) st = alloc_into(h, &h->gbase_dev, h->gdev_count * sizeof(double), "force schedule base");
+    // 64 copies of the force, up to 12 MB of them (every uniform force, and
+    // row forces of up to 8192 rows)
+    const size_t ring = 64 * (scale ? h->gdev_count : 3);
+    if (st == LBM_OK && ring <= (size_t)1 << 20) {
+        st = alloc_into(h, &h->gring_dev, ring * sizeof(double), "force schedule ring");
+        if (st == LBM_OK) st = alloc_into(h, &h->gring32_dev, ring * sizeof(float), "force schedule ring (FP32)");
+    }
     if (st != LBM_OK) {
         free_schedule(h);
         return st;
@@ -448,6 +559,8 @@ lbm_status handle_make_slab(lbm_handle *h, int ax, int g0, int gn) {
     h->kp.hg0 = g0;
     h->kp.hgn = gn;
     drop_graphs(h);
+    if (h->mask)
+        LBM_CUDA(h, launchers_for(h->lattice).links(h->kp, h->links_dev, nullptr, h->stream));
     return LBM_OK;
 }
 
@@ -481,6 +594,9 @@ void lbm_destroy(lbm_handle *h) {
     dev_free(h, h->gs_dev);
     dev_free(h, h->gbase_dev);
     dev_free(h, h->gs_t_dev);
+    dev_free(h, h->gring_dev);
+    dev_free(h, h->gring32_dev);
+    dev_free(h, h->links_dev);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete h;
 }
@@ -572,6 +688,7 @@ lbm_status lbm_create(const lbm_desc *d, lbm_handle **out) {
         h->cfg.bdx = 128;
     }
     h->graph_steps = 64;
+    h->fuse = true;   // where k_step_tile applies (tile_ok)
 
     lbm_status st;
     if (d->stream) {
@@ -641,6 +758,19 @@ lbm_status lbm_create(const lbm_desc *d, lbm_handle **out) {
             return s2;
         }
         kp.solid = h->solid_dev;
+        if ((st = alloc_into(h, &h->links_dev, (size_t)plane * sizeof(unsigned), "obstacle links")) != LBM_OK) {
+            std::string m = h->err;
+            lbm_destroy(h);
+            return fail(nullptr, st, m);
+        }
+        e = cudaMemsetAsync(h->links_dev, 0, (size_t)plane * sizeof(unsigned), h->stream);
+        if (e == cudaSuccess) e = launchers_for(h->lattice).links(kp, h->links_dev, nullptr, h->stream);
+        if (e != cudaSuccess) {
+            lbm_status s2 = cuda_fail(nullptr, e, "obstacle links");
+            lbm_destroy(h);
+            return s2;
+        }
+        kp.links = h->links_dev;
     }
     // initial state: target fbar in buffer B, unstreamed into buffer A
     double *rho0_dev = nullptr, *u0_dev = nullptr;
@@ -701,7 +831,11 @@ lbm_status lbm_step(lbm_handle *h, int64_t nsteps) {
             left -= h->graph_steps;
         }
     }
+    // into a caller's own capture, one step per launch: a replay of an even
+    // number of steps then ends in the buffer it began in
+    h->hold_fuse = cs != cudaStreamCaptureStatusNone;
     lbm_status st = launch_steps(h, left);
+    h->hold_fuse = false;
     if (st != LBM_OK) return st;
     h->step += nsteps;
     return LBM_OK;
@@ -851,6 +985,9 @@ lbm_status lbm_set_populations(lbm_handle *h, const double *f) {
     cudaError_t e = cudaMemcpyAsync(tmp, f, n * sizeof(double), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = L.put_pops(h->storage, h->kp, tmp, spare, h->stream);
     if (e == cudaSuccess) e = L.unstream(h->storage, h->mask, h->kp, spare, h->buf[h->cur], h->stream);
+    // the steps never write solid nodes: clear what the import left there, so
+    // that the raw state does not depend on which buffer a run ends in
+    if (e == cudaSuccess && h->mask) e = cudaMemsetAsync(spare, 0, h->state_bytes, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     dev_free(h, tmp);
     if (e != cudaSuccess) return cuda_fail(h, e, "population import");
@@ -894,7 +1031,14 @@ lbm_status lbm_set_launch_layout(lbm_handle *h, int block_x, int nodes_per_threa
     }
     LBM_CUDA(h, cudaStreamSynchronize(h->stream));
     h->cfg = c;
+    h->fuse = false;
     drop_graphs(h);
+    return LBM_OK;
+}
+
+lbm_status lbm_get_launch_steps(const lbm_handle *h, int *steps) {
+    if (!h || !steps) return fail(nullptr, LBM_ERR_ARG, "NULL argument");
+    *steps = fused_steps(h, 64);
     return LBM_OK;
 }
 
@@ -939,29 +1083,43 @@ lbm_status lbm_autotune(lbm_handle *h, int trials, int *block_x, int *nodes_per_
     }
     double best = 1e300;
     StepCfg best_cfg = h->cfg;
-    for (const StepCfg &c : shapes) {
+    // several steps per launch first (where it applies), then the shapes
+    h->fuse = true;
+    const int K = fused_steps(h, 64);
+    bool best_fused = false;
+    for (int v = K > 1 ? -1 : 0; v < (int)shapes.size(); ++v) {
+        const bool fused = v < 0;
+        const StepCfg c = fused ? h->cfg : shapes[v];
+        auto once = [&]() {
+            return fused ? launch_tile(h, K, h->g32_dev, 0, h->buf[h->cur], h->buf[1 - h->cur])
+                         : launch_step(h, c, h->buf[h->cur], h->buf[1 - h->cur]);
+        };
         // one untimed launch, then the timed ones; all read the state and
         // write the spare buffer
-        e = launch_step(h, c, h->buf[h->cur], h->buf[1 - h->cur]);
+        e = once();
         if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-        for (int t = 0; t < trials && e == cudaSuccess; ++t) e = launch_step(h, c, h->buf[h->cur], h->buf[1 - h->cur]);
+        for (int t = 0; t < trials && e == cudaSuccess; ++t) e = once();
         if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float t_ms = 0.f;
         if (e == cudaSuccess) e = cudaEventElapsedTime(&t_ms, e0, e1);
         if (e != cudaSuccess) break;
-        const double per = (double)t_ms / trials;
+        const double per = (double)t_ms / trials / (fused ? K : 1);
         if (per < best) {
             best = per;
             best_cfg = c;
+            best_fused = fused;
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (e != cudaSuccess) return cuda_fail(h, e, "autotune");
-    lbm_status st = lbm_set_launch_layout(h, best_cfg.bdx, best_cfg.npt,
-                                          best_cfg.vec ? LBM_LAYOUT_VECTOR : LBM_LAYOUT_STRIDED);
-    if (st != LBM_OK) return st;
+    drop_graphs(h);
+    if (!best_fused) {
+        lbm_status st = lbm_set_launch_layout(h, best_cfg.bdx, best_cfg.npt,
+                                              best_cfg.vec ? LBM_LAYOUT_VECTOR : LBM_LAYOUT_STRIDED);
+        if (st != LBM_OK) return st;
+    }
     if (block_x) *block_x = best_cfg.bdx;
     if (nodes_per_thread) *nodes_per_thread = best_cfg.npt;
     if (ms) *ms = best;
