@@ -17,6 +17,13 @@
 // scan is bounded by a no-progress counter that sets an error flag and exits.
 // Population data written during the kernel by other CTAs is read through L2
 // (ld.global.cg), never through the non-coherent read-only path.
+//
+// In FP32, steps without a residual check are taken two at a time: a tile is
+// then a run of kFuseX x kFuseY node tiles of the channel, each advanced by
+// two steps in shared memory (tile_steps of lbm_step_tile.cuh, bit for bit
+// the two single steps).  That halves the claims, the fences and the memory
+// traffic per step.  A channel's state moves to the other arena with every
+// claim's worth of steps, whether one or two (BatchCtl.flips).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,6 +33,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_internal.h"
+#include "lbm_step_tile.cuh"
 
 using namespace lbm;
 
@@ -44,6 +52,7 @@ struct BatchChan {
     long long solid_off; // offset of its obstacle mask and links (nxp * ny entries) in their arenas, -1: none
     int nx, ny, nxp;
     int per_x, per_y;
+    int fuse;            // takes kFuseSteps at a time (see fused_at)
     double om2, om3, om4;
     double gx, gy;
 };
@@ -66,6 +75,7 @@ struct BatchCtl {
     long long start;           // steps completed when the run began
     int status;
     double r;                  // last residual
+    int flips;                 // times the state moved to the other arena: it is in fa when even, in fb when odd
     int parked;                // 1: left the kernel at a step boundary for the handoff
 };
 
@@ -74,11 +84,12 @@ struct BatchRun {
     BatchCtl *ctl;
     int n;
     const unsigned *links;       // obstacle links of the channels with a mask
+    const float *g32;            // 4 values per channel
     int grid;                  // resident CTAs
     int tile_min, tile_max;    // nodes per tile
     long long *active_nodes;   // nodes of channels still running
     unsigned *active_bits;     // bit c: channel c still running
-    void *fa, *fb;  // the state after s steps lives in fa for even s, fb for odd s
+    void *fa, *fb;  // the two arenas (BatchCtl.flips)
     void *snap;
     double *part;
     int *active_count;
@@ -90,6 +101,20 @@ struct BatchRun {
     long long max_steps;   // per channel, counted from the run's start
     long long spin_limit;  // scans without any progress anywhere before giving up
 };
+
+// Tiles of the fused steps.  us per step of 128 channels (4.4 M nodes) at
+// blocks of 128 threads: 32 x 16 51, 30 x 14 56, 62 x 14 66, three steps of
+// 32 x 8 69; one step at a time, in row bands, 87.
+constexpr int kFuseSteps = 2, kFuseX = 32, kFuseY = 16;
+
+// whether a channel that started its run at step `start` takes kFuseSteps
+// steps at once from `step` on: none of them checks the residual (the steps
+// a multiple of K after the start do) or lies past the run's end
+__host__ __device__ inline bool fused_at(const BatchChan &C, long long step, long long start, int K, long long max_steps) {
+    if (!C.fuse) return false;
+    const long long done = step - start, r = done % K;
+    return r != 0 && r + kFuseSteps <= K && done + kFuseSteps <= max_steps;
+}
 
 template <typename T> __device__ __forceinline__ T ld_cg(const T *p);
 template <> __device__ __forceinline__ double ld_cg<double>(const double *p) { return __ldcg(p); }
@@ -205,21 +230,74 @@ __host__ __device__ inline int tiles_for(int nx, int ny, long long active, int g
     return (ny + rows - 1) / rows;
 }
 
+// Claims of a channel's next kFuseSteps steps: runs of node tiles, as many as
+// give every resident CTA one claim per round of all active channels (a claim
+// costs its CTA about 4 us of atomics and fences; measured for 128 channels,
+// us per step: runs of active / (2 grid) nodes 57, active / grid 51, twice that
+// 68, as CTAs then wait for a channel's last run).
+__device__ __forceinline__ int fused_tiles_for(const BatchChan &C, long long active, const BatchRun &r) {
+    const int subs = ((C.nx + kFuseX - 1) / kFuseX) * ((C.ny + kFuseY - 1) / kFuseY);
+    long long target = active / r.grid;
+    if (target < r.tile_min) target = r.tile_min;
+    if (target > 4LL * r.tile_max) target = 4LL * r.tile_max;
+    int run = (int)(target / (kFuseX * kFuseY));
+    const int min_run = (subs + kMaxTiles - 1) / kMaxTiles;
+    if (run < min_run) run = min_run;
+    if (run < 1) run = 1;
+    return (subs + run - 1) / run;
+}
+
+// The node tiles of claim `tile` of `ntiles`, advanced by kFuseSteps.  Out of
+// line: inlined, its registers made the claim loop and the single step spill
+// 180 bytes at the kernel's 64 registers.
+template <int COLL>
+__device__ __noinline__ void batch_fused(const BatchRun &r, int c, const float *fin, float *fout, int tile, int ntiles) {
+    extern __shared__ __align__(16) unsigned char batch_smem[];
+    const BatchChan &C = r.ch[c];
+    TileDom d;
+    d.nx = C.nx;
+    d.ny = C.ny;
+    d.nxp = C.nxp;
+    d.per_x = C.per_x;
+    d.per_y = C.per_y;
+    d.plane_bytes = (unsigned)(C.plane * sizeof(float));
+    d.links = C.solid_off >= 0 ? r.links + C.solid_off : nullptr;
+    d.force_kind = G_UNIFORM;
+    d.g = r.g32 + 4 * c;
+    d.g_step = 0;
+    d.g_plane = 0;
+    d.om2 = (float)C.om2;
+    d.om3 = (float)C.om3;
+    d.om4 = (float)C.om4;
+    d.omb = d.om2;
+    d.trim = false;   // the collision is the template's
+    const int nsx = (C.nx + kFuseX - 1) / kFuseX, subs = nsx * ((C.ny + kFuseY - 1) / kFuseY);
+    const int run = (subs + ntiles - 1) / ntiles;
+    const int end = min((tile + 1) * run, subs);
+    for (int t = tile * run; t < end; ++t) {
+        const int ty = t / nsx;
+        tile_steps<COLL, ST_F32, TILE_ANY_MASK, true, kFuseX, kFuseY, kFuseSteps, 0>(
+            d, fin, fout, reinterpret_cast<float *>(batch_smem), (t - ty * nsx) * kFuseX, ty * kFuseY);
+        __syncthreads();   // the next tile reuses the shared memory
+    }
+}
+
 // batch storage is FP32 or FP64 (loads through L2: ld.global.cg).  The
 // launch bounds cap the kernel at 64 registers (no spills in FP32), so 8
 // blocks of 128 threads share an SM instead of 6.
 template <int COLL, int ST>
-__global__ void __launch_bounds__(256, 4) k_batch(const BatchRun r) {
+__global__ void __launch_bounds__(256, 4) k_batch(const __grid_constant__ BatchRun r) {
     typedef typename Store<ST>::T T;
     typedef typename Store<ST>::R R;
-    __shared__ int s_c, s_tile, s_tiles, s_quit;
+    __shared__ int s_c, s_tile, s_tiles, s_quit, s_flips;
     __shared__ long long s_step;
     long long empty = 0;
     unsigned long long seen = 0;
     for (;;) {
         // warp 0 looks for a claimable tile: the active-channel bitmap is read
         // 32 words per load, the claim words of a word's channels in one round,
-        // and the lowest-index (highest-priority) claimable channel is claimed
+        // and a claimable channel of the first word that has one (the words
+        // are in priority order) is claimed
         if (threadIdx.x < 32) {
             const int lane = threadIdx.x;
             int fc = -1, ft = 0, fn = 0;
@@ -241,8 +319,11 @@ __global__ void __launch_bounds__(256, 4) k_batch(const BatchRun r) {
                     }
                     unsigned m = __ballot_sync(0xffffffffu, ok);
                     while (m != 0u) {
-                        const int pick = __ffs(m) - 1;
-                        m &= m - 1u;
+                        // CTAs start at different channels of the word: with
+                        // the lowest one first, all of them added to the same
+                        // few claim words and most came too late
+                        const int pick = (int)__fns(m, 0, 1 + (int)(blockIdx.x % (unsigned)__popc(m)));
+                        m &= ~(1u << pick);
                         unsigned long long w2 = 0ull;
                         if (lane == pick) w2 = atomicAdd(&r.ctl[c].claim, 1ull);
                         w2 = __shfl_sync(0xffffffffu, w2, pick);
@@ -281,6 +362,8 @@ __global__ void __launch_bounds__(256, 4) k_batch(const BatchRun r) {
                     empty = 0;
                 }
                 __threadfence();
+                // written before the claim word that opened these tiles
+                if (fc >= 0) s_flips = vload(&r.ctl[fc].flips);
             }
         }
         __syncthreads();
@@ -292,19 +375,31 @@ __global__ void __launch_bounds__(256, 4) k_batch(const BatchRun r) {
             const int tile = s_tile;
             const int ntiles = s_tiles;
             const int rows = (C.ny + ntiles - 1) / ntiles;
-            const T *fin = (const T *)((step & 1) ? r.fb : r.fa) + C.off;
-            T *fout = (T *)((step & 1) ? r.fa : r.fb) + C.off;
+            const int flips = s_flips;
+            const T *fin = (const T *)((flips & 1) ? r.fb : r.fa) + C.off;
+            T *fout = (T *)((flips & 1) ? r.fa : r.fb) + C.off;
             const long long start = r.ctl[c].start;
             const bool check = ((step - start) % r.K) == 0;
+            const bool fused = ST == ST_F32 && fused_at(C, step, start, r.K, r.max_steps);
             const int y0 = tile * rows;
             const int y1 = min(y0 + rows, C.ny);
-            const int nn = y1 > y0 ? (y1 - y0) * C.nx : 0;  // the last tiles may be empty
+            const int nn = !fused && y1 > y0 ? (y1 - y0) * C.nx : 0;  // the last tiles may be empty
             R *snap = (R *)r.snap + C.snap_off;
             const unsigned *links = C.solid_off >= 0 ? r.links + C.solid_off : nullptr;
             const int N = C.nx * C.ny;
             const R om2 = R(C.om2), om3 = R(C.om3), om4 = R(C.om4), gx = R(C.gx), gy = R(C.gy);
             const bool trim = C.om3 == 1.0 && C.om4 == 1.0;
             double v[2] = {0.0, 0.0};
+            if constexpr (ST == ST_F32) {
+                if (fused) {
+                    if constexpr (COLL == SMRT) {
+                        if (trim) batch_fused<SMRT_TRIM>(r, c, fin, fout, tile, ntiles);
+                        else batch_fused<SMRT>(r, c, fin, fout, tile, ntiles);
+                    } else {
+                        batch_fused<COLL>(r, c, fin, fout, tile, ntiles);
+                    }
+                }
+            }
             // two nodes per thread per pass, all loads issued first.  The
             // tile's nodes are numbered row by row; a thread's two nodes
             // (numbers base and base + blockDim.x) advance by 2 blockDim.x a
@@ -409,7 +504,7 @@ __global__ void __launch_bounds__(256, 4) k_batch(const BatchRun r) {
                 if (prev == (unsigned)(ntiles - 1)) {
                     // last tile of this step: close it
                     __threadfence();
-                    const long long done_steps = step + 1;
+                    const long long done_steps = step + (fused ? kFuseSteps : 1);
                     bool retire = false;
                     int status = 0;
                     if (check && step > start) {
@@ -433,6 +528,7 @@ __global__ void __launch_bounds__(256, 4) k_batch(const BatchRun r) {
                         status = r.tol >= 0.0 ? (int)LBM_NOT_CONVERGED : (int)LBM_OK;
                     }
                     r.ctl[c].steps = done_steps;
+                    r.ctl[c].flips = flips + 1;
                     atomicExch(&r.ctl[c].done, 0u);
                     // the tail: few channels left, each would take a whole
                     // scheduling round per step here; they leave at this step
@@ -447,7 +543,10 @@ __global__ void __launch_bounds__(256, 4) k_batch(const BatchRun r) {
                         atomicAdd((unsigned long long *)r.active_nodes, (unsigned long long)(-(long long)C.nx * C.ny));
                         atomicSub(r.active_count, 1);
                     } else {
-                        const int nt = tiles_for(C.nx, C.ny, vload(r.active_nodes), r.grid, r.tile_min, r.tile_max);
+                        const bool next_fused = ST == ST_F32 && fused_at(C, done_steps, start, r.K, r.max_steps);
+                        const long long active = vload(r.active_nodes);
+                        const int nt = next_fused ? fused_tiles_for(C, active, r)
+                                                  : tiles_for(C.nx, C.ny, active, r.grid, r.tile_min, r.tile_max);
                         __threadfence();
                         atomicExch(&r.ctl[c].claim, claim_word(done_steps, nt));
                     }
@@ -492,6 +591,7 @@ struct lbm_batch {
     std::vector<KParams> kp;    // per channel, pointing into the arenas
     std::vector<BatchChan> ch;
     std::vector<long long> steps;
+    std::vector<int> flips;     // which arena holds a channel's state (BatchCtl.flips)
     void *fa = nullptr, *fb = nullptr, *snap = nullptr;
     double *part = nullptr;
     double *g_dev = nullptr;    // per channel 4 doubles
@@ -597,13 +697,16 @@ lbm_status batch_run(lbm_batch *b, double tol, int K, int64_t max_steps) {
     int dev = 0, sms = 0, per_sm = 0;
     B_CUDA(b, cudaGetDevice(&dev));
     B_CUDA(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    B_CUDA(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, b->block, 0));
+    const size_t smem = b->storage == LBM_F32 ? TileGeo<kFuseX, kFuseY, kFuseSteps>::elems() * sizeof(float) : 0;
+    static_assert(TileGeo<kFuseX, kFuseY, kFuseSteps>::elems() * sizeof(float) <= 48 * 1024 - 256, "default shared memory");
+    B_CUDA(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, b->block, smem));
     if (per_sm < 1) return bfail(b, LBM_ERR_ARG, "batch block size does not fit on an SM");
     BatchRun r;
     r.ch = b->ch_dev;
     r.ctl = b->ctl_dev;
     r.n = b->n;
     r.links = b->links;
+    r.g32 = b->g32_dev;
     // at most 4000 CTAs: the tile field of the claim word overshoots the tile
     // count (<= 4096) by at most the number of concurrent claimers (< 8192 - 4096)
     r.grid = std::min(sms * per_sm, 4000);
@@ -630,7 +733,7 @@ lbm_status batch_run(lbm_batch *b, double tol, int K, int64_t max_steps) {
     B_CUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
     cudaMemsetAsync(b->active_bits, 0, (size_t)((b->n + 31) / 32) * 4, b->stream);
     k_batch_reset<<<(b->n + 127) / 128, 128, 0, b->stream>>>(r, b->total_nodes);
-    kern<<<grid, b->block, 0, b->stream>>>(r);
+    kern<<<grid, b->block, smem, b->stream>>>(r);
     cudaError_t e = cudaStreamEndCapture(b->stream, &g);
     if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("batch capture: ") + cudaGetErrorString(e));
     e = cudaGraphInstantiate(&ge, g, 0);
@@ -644,7 +747,10 @@ lbm_status batch_run(lbm_batch *b, double tol, int K, int64_t max_steps) {
     B_CUDA(b, bcopy(b, &errflag, b->error, sizeof(int), cudaMemcpyDeviceToHost));
     std::vector<BatchCtl> ctl(b->n);
     B_CUDA(b, bcopy(b, ctl.data(), b->ctl_dev, sizeof(BatchCtl) * b->n, cudaMemcpyDeviceToHost));
-    for (int c = 0; c < b->n; ++c) b->steps[c] = ctl[c].steps;
+    for (int c = 0; c < b->n; ++c) {
+        b->steps[c] = ctl[c].steps;
+        b->flips[c] = ctl[c].flips;
+    }
     if (errflag) return bfail(b, (lbm_status)errflag, "batch kernel stopped: no progress within the scan limit");
     return LBM_OK;
 }
@@ -664,6 +770,7 @@ lbm_status init_channels(lbm_batch *b) {
         if (e == cudaSuccess) e = L.unstream(b->storage, mask, b->kp[c], B, A, b->stream);
         if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, std::string("batch init: ") + cudaGetErrorString(e));
         b->steps[c] = 0;
+        b->flips[c] = 0;
         ctl[c] = BatchCtl{};
     }
     size_t snap_elems = 0;
@@ -676,7 +783,7 @@ lbm_status init_channels(lbm_batch *b) {
 
 const void *channel_state(const lbm_batch *b, int c) {
     const size_t eb = elem_bytes(b->storage);
-    return (const char *)((b->steps[c] & 1) ? b->fb : b->fa) + b->ch[c].off * eb;
+    return (const char *)((b->flips[c] & 1) ? b->fb : b->fa) + b->ch[c].off * eb;
 }
 
 // Continue the channels that parked in the tail of a run, each as a plain
@@ -804,8 +911,7 @@ lbm_status run_parked(lbm_batch *b, double tol, int K, int64_t max_steps) {
                 }
                 c.steps += 1;
             }
-            void *dst = (char *)((c.steps & 1) ? b->fb : b->fa) + b->ch[q.p].off * eb;
-            st = handle_export_state(q.h, dst);
+            st = handle_export_state(q.h, const_cast<void *>(channel_state(b, q.p)));
             e = st == LBM_OK ? cudaStreamSynchronize(handle_stream(q.h)) : cudaErrorUnknown;
             if (e != cudaSuccess) {
                 cleanup();
@@ -903,6 +1009,7 @@ lbm_status lbm_batch_create(const lbm_desc *descs, int n, lbm_batch **out) {
     b->ch.resize(n);
     b->kp.resize(n);
     b->steps.assign(n, 0);
+    b->flips.assign(n, 0);
     b->field_off.assign(n, 0);
     lbm_status st = LBM_OK;
     if (d0.stream) {
@@ -929,6 +1036,8 @@ lbm_status lbm_batch_create(const lbm_desc *descs, int n, lbm_batch **out) {
         parts += 2LL * d.ny;
         C.per_x = d.periodic[0] ? 1 : 0;
         C.per_y = d.periodic[1] ? 1 : 0;
+        // k_step_tile's conditions: wider than the margins, 32-bit byte offsets
+        C.fuse = d.nx > kFuseSteps && d.ny > kFuseSteps && 9 * C.plane * 4 < (1LL << 32) ? 1 : 0;
         C.om2 = 1.0 / d.tau[2];
         C.om3 = d.collision != LBM_BGK ? 1.0 / d.tau[3] : 0.0;
         C.om4 = d.collision != LBM_BGK ? 1.0 / d.tau[4] : 0.0;

@@ -94,10 +94,13 @@ template <int ST> __device__ __forceinline__ float one_at(const typename Store<S
     else return __bfloat162float(*p);
 }
 
-// step S of the tile at (X0, Y0): NT threads, all of them call it.  INNER: no
-// node of the tile or its margins, nor any source of theirs, lies across a
-// face of the domain, and there is no mask
-template <int COLL, int ST, bool MASK, bool CG, bool INNER, int TX, int TY, int K, int NT, int S>
+// Whether the domain has an obstacle mask: never, always, or when d.links is set
+enum { TILE_NO_MASK = 0, TILE_MASK = 1, TILE_ANY_MASK = 2 };
+
+// step S of the tile at (X0, Y0): NT threads (0: blockDim.x), all of them call
+// it.  INNER: no node of the tile or its margins, nor any source of theirs,
+// lies across a face of the domain, and there is no mask
+template <int COLL, int ST, int MASK, bool CG, bool INNER, int TX, int TY, int K, int NT, int S>
 __device__ __forceinline__ void tile_step(const TileDom &d, const typename Store<ST>::T *__restrict__ fin,
                                           typename Store<ST>::T *__restrict__ fout, typename Store<ST>::T *sm, int X0,
                                           int Y0) {
@@ -112,7 +115,7 @@ __device__ __forceinline__ void tile_step(const TileDom &d, const typename Store
         ugy = __ldg(g + 1);
     }
 #pragma unroll 1
-    for (int idx = threadIdx.x; idx < PW * H; idx += NT) {
+    for (int idx = threadIdx.x; idx < PW * H; idx += NT > 0 ? NT : (int)blockDim.x) {
         const int ry = idx / PW, rx = 2 * (idx - ry * PW);
         int x0 = X0 - M + rx, y = Y0 - M + ry;
         int xa = x0, xb = x0 + 1;
@@ -133,9 +136,9 @@ __device__ __forceinline__ void tile_step(const TileDom &d, const typename Store
             else if (xb >= d.nx) xb = d.per_x ? xb - d.nx : xa;
             ba = wall_bits(d, xa, y);
             bb = wall_bits(d, xb, y);
-            if constexpr (MASK) {
-                ba |= d.links[y * d.nxp + xa];
-                bb |= d.links[y * d.nxp + xb];
+            if (MASK == TILE_MASK || (MASK == TILE_ANY_MASK && d.links)) {
+                ba |= __ldg(d.links + y * d.nxp + xa);
+                bb |= __ldg(d.links + y * d.nxp + xb);
             }
         }
         F2 G[9];
@@ -206,7 +209,8 @@ __device__ __forceinline__ void tile_step(const TileDom &d, const typename Store
         } else {
             char *out = reinterpret_cast<char *>(fout);
             const unsigned q = ((unsigned)(y * d.nxp) + (unsigned)x0) * ES;
-            const bool sa = !MASK || (ba & 1u) == 0u, sb = INNER || (x0 + 1 < d.nx && (!MASK || (bb & 1u) == 0u));
+            // bit 0: a solid node
+            const bool sa = INNER || (ba & 1u) == 0u, sb = INNER || (x0 + 1 < d.nx && (bb & 1u) == 0u);
             if (sa && sb) {
                 static_for<9>([&](auto I) {
                     constexpr int i = decltype(I)::value;
@@ -225,7 +229,7 @@ __device__ __forceinline__ void tile_step(const TileDom &d, const typename Store
 }
 
 // all K steps of the tile at (X0, Y0)
-template <int COLL, int ST, bool MASK, bool CG, int TX, int TY, int K, int NT>
+template <int COLL, int ST, int MASK, bool CG, int TX, int TY, int K, int NT>
 __device__ __forceinline__ void tile_steps(const TileDom &d, const typename Store<ST>::T *__restrict__ fin,
                                            typename Store<ST>::T *__restrict__ fout, typename Store<ST>::T *sm, int X0,
                                            int Y0) {
@@ -236,10 +240,10 @@ __device__ __forceinline__ void tile_steps(const TileDom &d, const typename Stor
             tile_step<COLL, ST, MASK, CG, decltype(inner)::value != 0, TX, TY, K, NT, S>(d, fin, fout, sm, X0, Y0);
         });
     };
-    if constexpr (!MASK) {
+    if constexpr (MASK != TILE_MASK) {
         // most tiles of a large domain: the whole block takes the path
         // without wraps, walls and limits
-        if (X0 >= K && Y0 >= K && X0 + TX + K <= d.nx && Y0 + TY + K <= d.ny) {
+        if ((MASK == TILE_NO_MASK || !d.links) && X0 >= K && Y0 >= K && X0 + TX + K <= d.nx && Y0 + TY + K <= d.ny) {
             run(Idx<1>{});
             return;
         }
@@ -248,7 +252,7 @@ __device__ __forceinline__ void tile_steps(const TileDom &d, const typename Stor
 }
 
 // MINB blocks of NT threads per SM cap the registers at 64
-template <int COLL, int ST, bool MASK, int TX, int TY, int K, int NT, int MINB>
+template <int COLL, int ST, int MASK, int TX, int TY, int K, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_step_tile(const __grid_constant__ TileDom d,
                                                         const typename Store<ST>::T *__restrict__ fin,
                                                         typename Store<ST>::T *__restrict__ fout) {
@@ -265,7 +269,7 @@ template <int ST, bool MASK> struct TileDispatch {
         constexpr size_t smem = TileGeo<TX, TY, K>::elems() * sizeof(T);
         static_assert(smem <= 48 * 1024, "within the default dynamic shared memory");
         const dim3 grid((unsigned)((d.nx + TX - 1) / TX), (unsigned)((d.ny + TY - 1) / TY));
-        k_step_tile<COLL, ST, MASK, TX, TY, K, NT, MINB><<<grid, NT, smem, s>>>(d, (const T *)fin, (T *)fout);
+        k_step_tile<COLL, ST, MASK ? TILE_MASK : TILE_NO_MASK, TX, TY, K, NT, MINB><<<grid, NT, smem, s>>>(d, (const T *)fin, (T *)fout);
         return cudaGetLastError();
     }
     template <int COLL>

@@ -104,3 +104,31 @@ def test_autotune_keeps_the_state_and_a_valid_choice():
     _same(a, b, 9)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("coll", ["SMRT", "BGK", "SMRT_FNEQ", "MRT_RAW"])
+@pytest.mark.parametrize("K", [1, 2, 3, 7])
+def test_batch_pairs_of_steps_match_single_lattices(coll, K):
+    """Two steps at a time between the checks of a batched run: channels one node around the 32 x 16 tiles, too narrow
+    for pairs, with obstacles, and (SMRT) with and without the trimmed collision, over check intervals that leave
+    every remainder."""
+    import paper_2212_07494_gb300 as P
+    chans = []
+    for k, (nx, ny) in enumerate([(32, 16), (33, 17), (31, 15), (3, 9), (2, 3), (97, 40), (64, 33)]):
+        tau = (1.0, 1.0, 0.6 + 0.1 * k) + ((1.0, 1.0) if k % 2 else (0.9, 1.2))
+        ch = {"shape": (nx, ny, 1), "tau": tau, "periodic": (1, 0, 1), "g": [1e-5, 2e-6 * k]}
+        if k in (1, 5):
+            ch["solid"] = W.random_solid((nx, ny, 1), 40 + k, frac=0.1)
+        chans.append(ch)
+    b = P.Batch(chans, coll, "F32")
+    b.set_handoff(0)
+    for total, n in ((11, 11), (19, 8)):
+        b.run_to_steady(0.0, K, max_steps=n)
+        for i, ch in enumerate(chans):
+            assert b.info(i)[0] == total
+            gl = P.Lattice("D2Q9", coll, ch["shape"], ch["tau"], "F32", ch["periodic"], g=ch["g"], solid=ch.get("solid"))
+            gl.set_launch(64, 1)
+            gl.step(total)
+            assert np.array_equal(b.populations(i), gl.populations()), (i, total)
+            gl.close()
+    b.close()
