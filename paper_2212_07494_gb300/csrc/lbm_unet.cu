@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <string>
 #include <vector>
@@ -224,7 +225,7 @@ template <int BK> __device__ __forceinline__ int sw_off(int r, int c) {
     return r * sw_rowbytes<BK>() + ((c ^ x) << 4);
 }
 
-template <int BK> __device__ __forceinline__ uint64_t tc_desc_sw(unsigned saddr) {
+template <int BK> __host__ __device__ constexpr uint64_t tc_desc_sw(unsigned saddr) {
     constexpr unsigned SBO = 8 * sw_rowbytes<BK>();
     uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFF);
     d |= (uint64_t)1 << 16;                    // leading offset: unused by the swizzled K-major layout
@@ -881,6 +882,382 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(const WgTcArgs a, const __grid
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.ncol));
 }
 
+// k_conv_col: the convolution of up to 128 input channels on column tiles,
+// each CTA marching along x over a run of columns.  Of k_conv_tma's stage, one
+// barrier round and two copies cost the issuing thread about 400 clocks
+// (measured; a copy of 16 KB itself moves at 110 bytes per clock), every tile
+// fetched its column nine times and the weights nine times, and the epilogue's
+// lanes, a pixel each, stored and read their gate 16 bytes to a line: 40 - 75
+// us a full-resolution layer.  Here
+//  - a column is fetched once, (HB + 2) rows of NB images in the order
+//    [row][image], so that the shift dy of a tap is a shift of NB tile rows:
+//    the MMA's A descriptor starts (1 + dy) NB rows into the column.  The
+//    swizzle is a pattern of address bits, so a start inside an 8-row atom
+//    reads the same bytes the copy wrote;
+//  - the shift dx takes the neighbouring column, which the CTA has just used
+//    or will use next: a ring of columns in shared memory;
+//  - the weights stay in shared memory for the whole run (cin <= 64), or are
+//    streamed once per pair of columns (cin = 128);
+//  - the accumulators are double-buffered in TMEM.  Two warps issue the MMAs
+//    of alternate columns (an issue costs about 110 clocks, the MMA itself 41
+//    at N = 32 and 49 at N = 64, all measured), and two groups of four warps
+//    take alternate columns out, through shared memory: the gate's values
+//    arrive there by TMA and the results leave by TMA, clipped at the image's
+//    and the batch's end.
+// The MMAs of a column run in the order of k_conv_tma (tap, channel block,
+// 16-channel slice), so the sums are the same bits.  Rows past the image's end
+// or the batch's last image are zero-filled (or stale shared memory) and not
+// stored, so any H and batch fit.  Every wait is bounded, as in k_conv_tma;
+// after a failed one all loops run on without waiting.
+// us a launch, k_conv_tma and this kernel (128 x 256, batch 8, cold cache):
+// 32 -> 32 channels at full resolution 65 and 20, 32 -> 64 75 and 24, 64 -> 32
+// 41 and 21, 64 -> 64 at half resolution 39 and 13, 128 -> 128 at a quarter
+// 29 and 13, 128 -> 64 at half 63 and 16.
+struct ColArgs {
+    int HB, NB, ytiles, L, runs;  // tile rows, images per tile, tiles per column, columns per CTA, runs per row of tiles
+    int R, colb;                  // columns in the ring, bytes of one (BK channels)
+};
+constexpr int COL_WS = 5;         // weight stages when they are streamed
+constexpr int COL_RMAX = 8;
+
+__device__ __forceinline__ void mbar_init(unsigned long long *m, int count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(m)), "r"(count));
+}
+__device__ __forceinline__ void mbar_expect(unsigned long long *m, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(m)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned long long *m) {
+    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(m)) : "memory");
+}
+// One thread of a converged warp issues an MMA: accumulator acc (added to when
+// `more`), low words of the A and B descriptors, their common high word.  The
+// operands are computed from kernel parameters and block indices alone and no
+// wait's result steers the loop, so that they can stay in uniform registers,
+// which the instruction reads (a single lane issuing out of a diverged warp
+// took 120 - 150 clocks).
+__device__ __forceinline__ void mma_elect(unsigned acc, unsigned alo, unsigned blo, unsigned hi, uint32_t idesc,
+                                          unsigned more) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %3};\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t"
+        "}\n" ::"r"(acc),
+        "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(more));
+}
+__device__ __forceinline__ void commit_elect(unsigned mbar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t"
+        "}\n" ::"r"(mbar));
+}
+
+template <int BK, int NT, int CB, bool RES>
+__global__ void __launch_bounds__(384) k_conv_col(const ConvArgs a, const __grid_constant__ CUtensorMap tmA,
+                                                  const __grid_constant__ CUtensorMap tmB,
+                                                  const __grid_constant__ CUtensorMap tmY,
+                                                  const __grid_constant__ CUtensorMap tmG, const ColArgs c, int *err) {
+    constexpr unsigned WB = NT * BK * 2;    // one (tap, channel block) of the weights
+    constexpr int KB = 9 * CB;
+    constexpr int NW = RES ? 9 : COL_WS;    // weight barriers: one per tap, or one per stage
+    constexpr int NCOL = 2 * NT;            // TMEM columns: two accumulators
+    constexpr unsigned SB = 128 * NT * 2;   // an output tile: 128 rows of NT channels, swizzled
+    constexpr int OB = RES ? 2 : 1;         // output tiles per epilogue group
+    static_assert(NT == 32 || NT == 64, "an output row is one swizzle span");
+    extern __shared__ __align__(1024) unsigned char col_smem[];
+    __shared__ __align__(8) unsigned long long colfull[COL_RMAX], colempty[COL_RMAX], wfull[NW], wempty[NW], accfull[2],
+        accempty[2], gfull[2 * OB], gempty[2 * OB], done[2];
+    __shared__ unsigned tmem_base;
+    __shared__ volatile int s_fail;
+    __shared__ int s_cols, s_w, s_g;        // columns, weight blocks and gate tiles whose copies were issued
+    __shared__ float s_bias[NT];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    unsigned char *sm = (unsigned char *)(((uintptr_t)col_smem + 1023) & ~(uintptr_t)1023);
+    const unsigned scol = smem_addr(sm), sw = scol + (unsigned)(c.R * CB * c.colb),
+                   so = sw + (RES ? KB : COL_WS) * WB;
+    const int g = blockIdx.x / c.runs, x0 = (blockIdx.x - g * c.runs) * c.L;
+    const int len = min(c.L, a.W - x0);     // >= 1
+    const int yt = g % c.ytiles, ng = g / c.ytiles;
+    const int co0 = blockIdx.y * NT;
+    if (tid == 0) {
+        s_fail = 0;
+        s_cols = s_w = s_g = 0;
+        for (int i = 0; i < c.R; ++i) {
+            mbar_init(&colfull[i], 1);
+            mbar_init(&colempty[i], 2);     // both MMA warps
+        }
+        for (int i = 0; i < NW; ++i) {
+            mbar_init(&wfull[i], 1);
+            mbar_init(&wempty[i], 2);       // both MMA warps
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&accfull[i], 1);
+            mbar_init(&accempty[i], 128);
+            mbar_init(&done[i], 1);
+        }
+        for (int i = 0; i < 2 * OB; ++i) {
+            mbar_init(&gfull[i], 1);
+            mbar_init(&gempty[i], 1);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;");
+        mbar_arrive(&colempty[0]);          // column 0 has one user only
+    }
+    if (tid >= 128 && tid < 128 + NT) s_bias[tid - 128] = a.bias ? a.bias[co0 + tid - 128] : 0.f;
+    if (warp == 2) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base)),
+                     "r"(NCOL));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const unsigned tmem = tmem_base;
+    // the gate's tile of column i into the output tile that column i will leave from
+    auto gate_load = [&](int i) {
+        const int k = i >> 1, b = (i & 1) * OB + k % OB;
+        if (k >= OB && !ws_wait(&gempty[b], (k / OB - 1) & 1, &s_fail)) return false;
+        mbar_expect(&gfull[b], (unsigned)(c.HB * c.NB * NT * 2));
+        tma_load4(so + b * SB, &tmG, co0, x0 + i, ng * c.NB, yt * c.HB, smem_addr(&gfull[b]));
+        s_g = i + 1;
+        return true;
+    };
+    if (warp == 0) {
+        if (lane == 0) {
+            // ---- columns x0 - 1 .. x0 + len
+            const unsigned bytes = (unsigned)((c.HB + 2) * c.NB * BK * 2) * CB;
+            int s = 0, ph = 1;              // ring slot, parity of its previous release
+            for (int j = 0; j < len + 2; ++j) {
+                if (j >= c.R && !ws_wait(&colempty[s], ph, &s_fail)) break;
+                int x = x0 - 1 + j;
+                if (a.wrapx) x = x < 0 ? x + a.W : (x >= a.W ? x - a.W : x);
+                mbar_expect(&colfull[s], bytes);
+#pragma unroll
+                for (int cb = 0; cb < CB; ++cb)
+                    tma_load4(scol + (unsigned)((s * CB + cb) * c.colb), &tmA, cb * BK, x, ng * c.NB, yt * c.HB - 1,
+                              smem_addr(&colfull[s]));
+                s_cols = j + 1;
+                if (++s == c.R) {
+                    s = 0;
+                    ph ^= 1;
+                }
+                if (!RES && a.gate && j >= 2 && !gate_load(j - 2)) break;
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            // ---- weights
+            const int n = RES ? KB : (len + 1) / 2 * KB;
+            int kb = 0, s = 0, ph = 1;
+            for (int k = 0; k < n; ++k) {
+                if (!RES && k >= COL_WS && !ws_wait(&wempty[s], ph, &s_fail)) break;
+                const int tap = kb / CB, cb = kb - tap * CB;
+                unsigned long long *bar = &wfull[RES ? tap : s];
+                if (RES) {
+                    if (cb == 0) mbar_expect(bar, CB * WB);
+                } else {
+                    mbar_expect(bar, WB);
+                }
+                asm volatile(
+                    "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                    "[%4];" ::"r"(sw + (unsigned)(RES ? kb : s) * WB),
+                    "l"(reinterpret_cast<uint64_t>(&tmB)), "r"(tap * a.cin + cb * BK), "r"(co0), "r"(smem_addr(bar))
+                    : "memory");
+                s_w = k + 1;
+                if (++kb == KB) kb = 0;
+                if (++s == COL_WS) {
+                    s = 0;
+                    ph ^= 1;
+                }
+            }
+            if (RES && a.gate)
+                for (int i = 0; i < len && gate_load(i); ++i) {}
+        }
+    } else if (warp < 4) {
+        // ---- MMA issuers: warp 2 takes the even columns, warp 3 the odd ones.
+        // Streamed weights serve a pair of columns: both warps go through
+        // every stage, a warp without a column (an odd last one) just
+        // releases it
+        constexpr uint32_t IDESC = tc_idesc(128, NT);
+        constexpr unsigned HI = (unsigned)(tc_desc_sw<BK>(0) >> 32);
+        const int me = warp - 2;
+        // descriptor words of addresses: 16-byte units
+        const unsigned row16 = (unsigned)(c.NB * BK * 2) >> 4;      // one row y: NB tile rows
+        const unsigned colb16 = (unsigned)(CB * c.colb) >> 4, cb16 = (unsigned)c.colb >> 4;
+        const unsigned c16 = (scol >> 4) | (1u << 16), w16 = (sw >> 4) | (1u << 16);
+        const unsigned acc = tmem + (unsigned)(me * NT);
+        int s0 = me, s1 = me + 1, s2 = me + 2, p1 = 0, p2 = 0;      // ring slots of columns i, i + 1, i + 2, and phases
+        if (s2 == c.R) {
+            s2 = 0;
+            p2 = 1;
+        }
+        int ws = 0, wph = 0;
+        const int end = RES ? len : (len + 1) / 2 * 2;
+        ws_wait(&colfull[s0], 0, &s_fail);                          // later ones were waited for as a column i + 2
+        for (int i = me; i < end; i += 2) {
+            const bool active = RES || i < len;
+            if (active) {
+                ws_wait(&colfull[s1], p1, &s_fail);
+                ws_wait(&colfull[s2], p2, &s_fail);
+                if (i >= 2) ws_wait(&accempty[me], ((i >> 1) - 1) & 1, &s_fail);
+                asm volatile("tcgen05.fence::after_thread_sync;");
+            }
+            const unsigned col0 = c16 + s0 * colb16, col1 = c16 + s1 * colb16, col2 = c16 + s2 * colb16;
+            // rolled: a CTA passes here once per column, a few times in all, and
+            // unrolled over the taps most of its time went into fetching
+            // instructions (1400 clocks a stage on the first pass, 330 after)
+            unsigned row = 0;
+            int dx = 0;
+#pragma unroll 1
+            for (int tap = 0; tap < 9; ++tap) {
+                const unsigned a16 = (dx == 0 ? col0 : (dx == 1 ? col1 : col2)) + row;
+                if (++dx == 3) {
+                    dx = 0;
+                    row += row16;
+                }
+                if (RES && i == me) ws_wait(&wfull[tap], 0, &s_fail);
+#pragma unroll 1
+                for (int cb = 0; cb < CB; ++cb) {
+                    if (!RES) ws_wait(&wfull[ws], wph, &s_fail);
+                    const unsigned a0 = a16 + cb * cb16, b0 = w16 + (unsigned)(RES ? tap * CB + cb : ws) * (WB >> 4);
+                    if (active)
+#pragma unroll
+                        for (int ks = 0; ks < BK / 16; ++ks)
+                            mma_elect(acc, a0 + 2 * ks, b0 + 2 * ks, HI, IDESC, ks > 0 ? 1u : (unsigned)(tap + cb));
+                    if (!RES) {
+                        commit_elect(smem_addr(&wempty[ws]));
+                        if (++ws == COL_WS) {
+                            ws = 0;
+                            wph ^= 1;
+                        }
+                    }
+                }
+            }
+            if (active) {
+                // column i is not used again by this warp, nor (its next one
+                // is i + 2) column i + 1
+                commit_elect(smem_addr(&accfull[me]));
+                commit_elect(smem_addr(&colempty[s0]));
+                commit_elect(smem_addr(&colempty[s1]));
+            }
+            s0 = s2;
+            s1 = s2 + 1;
+            p1 = p2;
+            if (s1 == c.R) {
+                s1 = 0;
+                p1 ^= 1;
+            }
+            s2 = s1 + 1;
+            p2 = p1;
+            if (s2 == c.R) {
+                s2 = 0;
+                p2 ^= 1;
+            }
+        }
+        // completes when every MMA this warp issued has
+        commit_elect(smem_addr(&done[me]));
+    } else {
+        // ---- epilogue: group (warp - 4) / 4 takes every second column
+        const int grp = (warp - 4) >> 2, q = warp & 3;
+        const int r = q * 32 + lane;            // tile row: image r % NB of row r / NB
+        const bool row = r < c.HB * c.NB;
+        const bool leader = (tid & 127) == 0;
+        for (int i = grp; i < len; i += 2) {
+            const int k = i >> 1, b = grp * OB + k % OB;
+            unsigned char *stage = sm + (so - scol) + b * SB;
+            ws_wait(&accfull[grp], k & 1, &s_fail);
+            if (a.gate) ws_wait(&gfull[b], (k / OB) & 1, &s_fail);
+            __syncwarp();
+            asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+            for (int ch = 0; ch < NT; ch += 32) {
+                unsigned v[32];
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+                    "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+                      "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
+                      "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
+                      "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+                    : "r"(tmem + (unsigned)(grp * NT + ch) + ((unsigned)(q * 32) << 16)));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                if (ch + 32 == NT) {
+                    asm volatile("tcgen05.fence::before_thread_sync;");
+                    mbar_arrive(&accempty[grp]);
+                }
+                if (row) {
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {   // 8 channels, 16 bytes, at a time
+                        uint4 *at = reinterpret_cast<uint4 *>(stage + sw_off<NT>(r, ch / 8 + h));
+                        uint4 gv = make_uint4(0u, 0u, 0u, 0u);
+                        if (a.gate) gv = *at;       // where the result goes
+                        const __nv_bfloat162 *gb = reinterpret_cast<const __nv_bfloat162 *>(&gv);
+                        __align__(16) __nv_bfloat162 o[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int e = 8 * h + 2 * k;
+                            float lo = __uint_as_float(v[e]) + s_bias[ch + e];
+                            float hi = __uint_as_float(v[e + 1]) + s_bias[ch + e + 1];
+                            if (a.relu) {
+                                lo = fmaxf(lo, 0.f);
+                                hi = fmaxf(hi, 0.f);
+                            }
+                            if (a.gate) {
+                                const float2 f = __bfloat1622float2(gb[k]);
+                                if (!(f.x > 0.f)) lo = 0.f;
+                                if (!(f.y > 0.f)) hi = 0.f;
+                            }
+                            o[k] = __floats2bfloat162_rn(lo, hi);
+                        }
+                        *at = *reinterpret_cast<const uint4 *>(o);
+                    }
+                }
+                __syncwarp();
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
+            if (leader) {
+                if (!s_fail) {
+                    asm volatile(
+                        "cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
+                            reinterpret_cast<uint64_t>(&tmY)),
+                        "r"(co0), "r"(x0 + i), "r"(ng * c.NB), "r"(yt * c.HB), "r"(so + b * SB)
+                        : "memory");
+                }
+                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                // the store OB - 1 columns back has read its tile: the next
+                // column's gate and results may overwrite it
+                asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(OB - 1) : "memory");
+                if (k >= OB - 1) mbar_arrive(&gempty[grp * OB + (k - (OB - 1)) % OB]);
+            }
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
+        }
+        if (leader) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    if (tid == 0 && s_fail) {
+        // issued copies land and issued MMAs finish before the CTA frees its
+        // TMEM and leaves: the last copy into every buffer, and all MMAs
+        volatile int never = 0;
+        for (int j = max(0, s_cols - c.R); j < s_cols; ++j) ws_wait(&colfull[j % c.R], (j / c.R) & 1, &never);
+        for (int i = max(0, s_g - 2 * OB); i < s_g; ++i) ws_wait(&gfull[(i & 1) * OB + (i >> 1) % OB], ((i >> 1) / OB) & 1, &never);
+        if (RES) {
+            for (int t = 0; t * CB < s_w; ++t) ws_wait(&wfull[t], 0, &never);
+        } else {
+            for (int k = max(0, s_w - COL_WS); k < s_w; ++k) ws_wait(&wfull[k % COL_WS], (k / COL_WS) & 1, &never);
+        }
+        ws_wait(&done[0], 0, &never);
+        ws_wait(&done[1], 0, &never);
+        atomicExch(err, 1);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NCOL));
+}
+
 // ------------------------------------------------------------- small kernels
 // bias gradient: db[c] += sum_p dz[p][c].  A block of 256 threads takes all
 // C channels of a chunk of pixels.  Thread t reads the 8 channels of group
@@ -1226,6 +1603,89 @@ template <int BK, int NT> bool launch_tma(lbm_unet *u, const ConvArgs &a, lbm_st
     return true;
 }
 
+// The column convolution where its operands fit shared memory (cin 16, 32, 64
+// or 128) and every global address and stride is a multiple of 16 bytes;
+// returns false (nothing launched) otherwise.  Each CTA takes one run of
+// columns, about tiles / SMs of them, and up to 64 output channels.
+template <int BK, int NT, int CB, bool RES>
+bool launch_col(lbm_unet *u, const ConvArgs &a, lbm_status *st) {
+    const int H = a.H, W = a.W, N = a.N;
+    ColArgs c{};
+    c.HB = H <= 128 ? H : 128;
+    c.NB = std::max(1, 128 / c.HB);
+    c.ytiles = (H + c.HB - 1) / c.HB;
+    const int groups = c.ytiles * ((N + c.NB - 1) / c.NB), nblocks = a.cout / NT;
+    const long long tiles = (long long)groups * W * nblocks;
+    c.L = (int)std::min<long long>(W, (tiles + u->sms - 1) / u->sms);
+    c.runs = (W + c.L - 1) / c.L;
+    // a slot holds what the MMAs of any tap may read: 128 rows from (1 + dy) NB on
+    c.colb = ((128 + 2 * c.NB) * BK * 2 + 1023) / 1024 * 1024;
+    constexpr size_t WB = (size_t)NT * BK * 2;
+    const size_t wbytes = (RES ? 9 * CB : COL_WS) * WB, obytes = (RES ? 4 : 2) * 128 * NT * 2, room = 232448 - 2048 - wbytes - obytes;
+    c.R = (int)std::min<size_t>({(size_t)COL_RMAX, (size_t)(c.L + 2), room / ((size_t)CB * c.colb)});
+    if (c.R < 3 || (!RES && c.L > 1 && c.R < 4)) return false;   // streamed weights: a pair's four columns at once
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tmap_encoder();
+    if (!enc) return false;
+    auto swz = [](int ch) {
+        return ch == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : (ch == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+    };
+    // NHWC activations as (channel, x, image, y), so that a box is laid out [y][image][channel]
+    auto image = [&](CUtensorMap *m, const bf16 *p, int ch, int stride, int boxc, int rows) {
+        const cuuint32_t es[4] = {1u, 1u, 1u, 1u};
+        const cuuint64_t pix = (cuuint64_t)stride * 2;
+        const cuuint64_t gd[4] = {(cuuint64_t)ch, (cuuint64_t)W, (cuuint64_t)N, (cuuint64_t)H};
+        const cuuint64_t gs[3] = {pix, pix * W * H, pix * W};
+        const cuuint32_t box[4] = {(cuuint32_t)boxc, 1u, (cuuint32_t)c.NB, (cuuint32_t)rows};
+        return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)p, gd, gs, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   swz(boxc), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    alignas(64) CUtensorMap ta, tb, ty, tg;
+    const cuuint32_t es[2] = {1u, 1u};
+    const cuuint64_t gdB[2] = {(cuuint64_t)9 * a.cin, (cuuint64_t)a.wrows};
+    const cuuint64_t gsB[1] = {(cuuint64_t)9 * a.cin * 2};
+    const cuuint32_t boxB[2] = {(cuuint32_t)BK, (cuuint32_t)NT};
+    if (!image(&ta, a.x + a.xo, a.cin, a.xc, BK, c.HB + 2) || !image(&ty, a.y + a.yo, a.cout, a.yc, NT, c.HB) ||
+        !image(&tg, a.gate ? a.gate + a.go : a.y + a.yo, a.cout, a.gate ? a.gc : a.yc, NT, c.HB) ||
+        enc(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)a.w, gdB, gsB, boxB, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            swz(BK), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+    // resident CTAs must not need more than an SM's 512 TMEM columns
+    const size_t need = (size_t)c.R * CB * c.colb + wbytes + obytes + 1024, floor_ = 233472 / (512 / (2 * NT) + 1) - 1024 + 1;
+    const size_t smem = std::max(need, floor_);
+    static bool attr = false;
+    cudaError_t e = cudaSuccess;
+    if (!attr) {
+        e = cudaFuncSetAttribute(k_conv_col<BK, NT, CB, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 1024);
+        attr = e == cudaSuccess;
+    }
+    if (e == cudaSuccess) {
+        k_conv_col<BK, NT, CB, RES><<<dim3((unsigned)(groups * c.runs), (unsigned)nblocks), 384, smem, u->stream>>>(
+            a, ta, tb, ty, tg, c, u->tc_err);
+        e = cudaGetLastError();
+    }
+    *st = e == cudaSuccess ? LBM_OK : ufail(u, LBM_ERR_CUDA, std::string("k_conv_col: ") + cudaGetErrorString(e));
+    return true;
+}
+
+bool conv_col(lbm_unet *u, const ConvArgs &a, lbm_status *st) {
+    auto al = [](const void *p) { return (uintptr_t)p % 16 == 0; };
+    if (a.cin > 128 || a.xc % 8 || a.xo % 8 || a.yc % 8 || a.yo % 8 || !al(a.x) || !al(a.w) || !al(a.y) || !a.y ||
+        (a.gate && (a.gc % 8 || a.go % 8 || !al(a.gate))))
+        return false;
+    if (a.cin == 128) {
+        if (a.cout % 64 == 0) return launch_col<64, 64, 2, false>(u, a, st);
+    } else if (a.cin == 64) {
+        if (a.cout % 64 == 0) return launch_col<64, 64, 1, true>(u, a, st);
+        if (a.cout == 32) return launch_col<64, 32, 1, true>(u, a, st);
+    } else if (a.cin == 32) {
+        if (a.cout % 64 == 0) return launch_col<32, 64, 1, true>(u, a, st);
+        if (a.cout == 32) return launch_col<32, 32, 1, true>(u, a, st);
+    } else if (a.cin == 16) {
+        if (a.cout == 32) return launch_col<16, 32, 1, true>(u, a, st);
+    }
+    return false;
+}
+
 template <int BK> lbm_status launch_conv_n(lbm_unet *u, const ConvArgs &a, long long M) {
     lbm_status st = LBM_OK;
     if (a.cout <= 16) return launch_tma<BK, 16>(u, a, &st) ? st : launch_tc<BK, 16>(u, a, M);
@@ -1237,6 +1697,8 @@ template <int BK> lbm_status launch_conv_n(lbm_unet *u, const ConvArgs &a, long 
 // convolutions with N = cout a multiple of 16 (every layer but the head):
 // TMA-fed where the shape allows, else cp.async-fed
 lbm_status conv_tc(lbm_unet *u, const ConvArgs &a, long long M) {
+    lbm_status st = LBM_OK;
+    if (conv_col(u, a, &st)) return st;
     if (a.cin % 64 == 0) return launch_conv_n<64>(u, a, M);
     if (a.cin % 32 == 0) return launch_conv_n<32>(u, a, M);
     return launch_conv_n<16>(u, a, M);
