@@ -1188,7 +1188,16 @@ __global__ void __launch_bounds__(384) k_conv_col(const ConvArgs a, const __grid
                     asm volatile("tcgen05.fence::before_thread_sync;");
                     mbar_arrive(&accempty[grp]);
                 }
-                if (row) {
+                if (a.yf) {
+                    // the head: yfc FP32 channels per pixel, straight to memory
+                    const int n = ng * c.NB + r % c.NB, y = yt * c.HB + r / c.NB;
+                    if (ch == 0 && row && n < a.N && y < a.H) {
+                        float *dst = a.yf + (((long long)n * a.H + y) * a.W + x0 + i) * a.yfc;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (e < a.yfc) dst[e] = __uint_as_float(v[e]) + s_bias[e];
+                    }
+                } else if (row) {
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {   // 8 channels, 16 bytes, at a time
                         uint4 *at = reinterpret_cast<uint4 *>(stage + sw_off<NT>(r, ch / 8 + h));
@@ -1220,7 +1229,7 @@ __global__ void __launch_bounds__(384) k_conv_col(const ConvArgs a, const __grid
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
             if (leader) {
-                if (!s_fail) {
+                if (!s_fail && !a.yf) {
                     asm volatile(
                         "cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
                             reinterpret_cast<uint64_t>(&tmY)),
@@ -1266,7 +1275,7 @@ __global__ void __launch_bounds__(384) k_conv_col(const ConvArgs a, const __grid
 // shared memory and each channel's sum goes out in one atomic.  Channels
 // C .. 8 G - 1 are read (the buffer has them: its stride is a multiple of 8)
 // but never written.
-constexpr int kBiasLoads = 16;  // loads per thread and block
+constexpr int kBiasLoads = 8;   // loads per thread and block, all in flight at once
 __global__ void __launch_bounds__(256) k_bias_grad(const bf16 *dz, int dzc, int C, long long P, int chunk, float *db) {
     __shared__ float sh[256 * 8];
     const int G = (C + 7) >> 3, R = 256 / G;
@@ -1275,9 +1284,15 @@ __global__ void __launch_bounds__(256) k_bias_grad(const bf16 *dz, int dzc, int 
     const long long p1 = p0 + chunk < P ? p0 + chunk : P;
     if (r < R) {
         float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (long long p = p0 + r; p < p1; p += R) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(dz + p * dzc + g * 8);
-            const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
+        uint4 v[kBiasLoads];
+#pragma unroll
+        for (int q = 0; q < kBiasLoads; ++q) {
+            const long long p = p0 + r + (long long)q * R;
+            v[q] = p < p1 ? __ldg(reinterpret_cast<const uint4 *>(dz + p * dzc + g * 8)) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int q = 0; q < kBiasLoads; ++q) {
+            const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v[q]);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const float2 f = __bfloat1622float2(h[k]);
@@ -1296,38 +1311,67 @@ __global__ void __launch_bounds__(256) k_bias_grad(const bf16 *dz, int dzc, int 
     }
 }
 
-// 2x2 average pooling: y[n][i][j] = mean of x[n][2i..2i+1][2j..2j+1]
-__global__ void k_pool(const bf16 *x, int xc, int xo, bf16 *y, int yc, int yo, int N, int H, int W, int C) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int Ho = H / 2, Wo = W / 2;
-    const long long total = (long long)N * Ho * Wo * C;
-    if (idx >= total) return;
-    const int c = (int)(idx % C);
-    const long long q = idx / C;
-    const int j = (int)(q % Wo), i = (int)((q / Wo) % Ho), n = (int)(q / ((long long)Wo * Ho));
-    auto at = [&](int yy, int xx) {
-        return __bfloat162float(x[((long long)(n * H + yy) * W + xx) * xc + xo + c]);
-    };
-    const float s = 0.25f * (at(2 * i, 2 * j) + at(2 * i, 2 * j + 1) + at(2 * i + 1, 2 * j) + at(2 * i + 1, 2 * j + 1));
-    y[((long long)(n * Ho + i) * Wo + j) * yc + yo + c] = __float2bfloat16_rn(s);
+// The pooling and upsampling kernels: a thread takes 8 channels (16 bytes; all
+// channel counts, strides and offsets are multiples of 8) of one pixel, a grid
+// row (blockIdx.y) one image row, so that no element needs a 64-bit division.
+// One channel per thread they were bound by those: full-resolution
+// pool_back 54 us, up_back 30, pool 18; now 12, 9 and 9 (128 x 256, batch 8).
+__device__ __forceinline__ void unpack8(const uint4 &v, float (&f)[8]) {
+    const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float2 t = __bfloat1622float2(h[k]);
+        f[2 * k] = t.x;
+        f[2 * k + 1] = t.y;
+    }
+}
+__device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
+    __align__(16) __nv_bfloat162 h[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) h[k] = __floats2bfloat162_rn(f[2 * k], f[2 * k + 1]);
+    return *reinterpret_cast<const uint4 *>(h);
+}
+__device__ __forceinline__ uint4 ld8(const bf16 *p) { return __ldg(reinterpret_cast<const uint4 *>(p)); }
+
+// 2x2 average pooling: y[n][i][j] = mean of x[n][2i..2i+1][2j..2j+1]; H, W:
+// fine sizes, grid (ceil(W/2 * C/8 / 256), N * H/2)
+__global__ void k_pool(const bf16 *x, int xc, int xo, bf16 *y, int yc, int yo, int H, int W, int C) {
+    const int C8 = C >> 3, Wo = W >> 1, Ho = H >> 1;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= Wo * C8) return;
+    const int row = blockIdx.y, n = row / Ho, i = row - n * Ho;
+    const int j = t / C8, c = (t - j * C8) * 8;
+    const bf16 *p = x + ((long long)(n * H + 2 * i) * W + 2 * j) * xc + xo + c;
+    float a[8], b[8], d[8], e[8];
+    unpack8(ld8(p), a);
+    unpack8(ld8(p + xc), b);
+    unpack8(ld8(p + (long long)W * xc), d);
+    unpack8(ld8(p + (long long)W * xc + xc), e);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) a[k] = 0.25f * (a[k] + b[k] + d[k] + e[k]);
+    *reinterpret_cast<uint4 *>(y + ((long long)row * Wo + j) * yc + yo + c) = pack8(a);
 }
 
-// pooling backward at the fine resolution, gated by the fine activation:
-// dst[n][y][x][c] (+)= 0.25 dy[n][y/2][x/2][c] * (gate > 0)
+// pooling backward at the fine resolution, gated by the fine activation and
+// added to dst: dst[n][y][x][c] += 0.25 dy[n][y/2][x/2][c] * (gate > 0); grid
+// (ceil(W * C/8 / 256), N * H)
 __global__ void k_pool_back(const bf16 *dy, int dyc, int dyo, const bf16 *gate, int gc, int go, bf16 *dst, int dc, int dof,
-                            int N, int H, int W, int C, int accumulate) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = (long long)N * H * W * C;
-    if (idx >= total) return;
-    const int c = (int)(idx % C);
-    const long long p = idx / C;
-    const int x = (int)(p % W), yv = (int)((p / W) % H), n = (int)(p / ((long long)W * H));
-    const long long pc = ((long long)(n * (H / 2) + yv / 2) * (W / 2) + x / 2);
-    float v = 0.25f * __bfloat162float(dy[pc * dyc + dyo + c]);
-    if (!(__bfloat162float(gate[p * gc + go + c]) > 0.f)) v = 0.f;
-    bf16 *d = dst + p * dc + dof + c;
-    if (accumulate) v += __bfloat162float(*d);
-    *d = __float2bfloat16_rn(v);
+                            int H, int W, int C) {
+    const int C8 = C >> 3;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= W * C8) return;
+    const int row = blockIdx.y, n = row / H, yv = row - n * H;
+    const int x = t / C8, c = (t - x * C8) * 8;
+    const long long p = (long long)row * W + x;
+    const long long pc = (long long)(n * (H / 2) + yv / 2) * (W / 2) + x / 2;
+    uint4 *d = reinterpret_cast<uint4 *>(dst + p * dc + dof + c);
+    float v[8], g[8], o[8];
+    unpack8(ld8(dy + pc * dyc + dyo + c), v);
+    unpack8(ld8(gate + p * gc + go + c), g);
+    unpack8(*d, o);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) o[k] = (g[k] > 0.f ? 0.25f * v[k] : 0.f) + o[k];
+    *d = pack8(o);
 }
 
 // nearest 2x upsampling: y[n][i][j] = x[n][i/2][j/2]
@@ -1345,80 +1389,144 @@ __global__ void k_up(const bf16 *x, int xc, int xo, bf16 *y, int yc, int yo, int
     *reinterpret_cast<uint4 *>(y + p * yc + yo + c) = *reinterpret_cast<const uint4 *>(x + q * xc + xo + c);
 }
 
-// upsampling backward at the coarse resolution, gated by the coarse activation
+// upsampling backward at the coarse resolution, gated by the coarse
+// activation; H, W: coarse sizes, grid (ceil(W * C/8 / 256), N * H)
 __global__ void k_up_back(const bf16 *dy, int dyc, int dyo, const bf16 *gate, int gc, int go, bf16 *dst, int dc, int dof,
-                          int N, int H, int W, int C) {
-    // H, W: coarse sizes
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = (long long)N * H * W * C;
-    if (idx >= total) return;
-    const int c = (int)(idx % C);
-    const long long p = idx / C;
-    const int j = (int)(p % W), i = (int)((p / W) % H), n = (int)(p / ((long long)W * H));
-    const int W2 = 2 * W, H2 = 2 * H;
-    float s = 0.f;
+                          int H, int W, int C) {
+    const int C8 = C >> 3;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= W * C8) return;
+    const int row = blockIdx.y, j = t / C8, c = (t - j * C8) * 8;
+    const long long p = (long long)row * W + j;
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, g[8];
+    unpack8(ld8(gate + p * gc + go + c), g);
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int b = 0; b < 2; ++b)
-            s += __bfloat162float(dy[((long long)(n * H2 + 2 * i + a) * W2 + 2 * j + b) * dyc + dyo + c]);
-    if (!(__bfloat162float(gate[p * gc + go + c]) > 0.f)) s = 0.f;
-    dst[p * dc + dof + c] = __float2bfloat16_rn(s);
+        for (int b = 0; b < 2; ++b) {
+            float v[8];
+            unpack8(ld8(dy + ((2LL * row + a) * (2 * W) + 2 * j + b) * dyc + dyo + c), v);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s[k] += v[k];
+        }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        if (!(g[k] > 0.f)) s[k] = 0.f;
+    *reinterpret_cast<uint4 *>(dst + p * dc + dof + c) = pack8(s);
 }
 
-// inputs [p][cin] FP32 -> [p][16] BF16 (channels cin..15 zero), cin <= 16
+// inputs [p][cin] FP32 -> [p][16] BF16 (channels cin..15 zero), cin <= 16;
+// two threads per pixel, 8 channels (16 bytes) each
 __global__ void k_pack_input(const float *x, int cin, bf16 *y, long long P) {
-    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P) return;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 2 * P) return;
+    const long long p = i >> 1;
+    const int c0 = (int)(i & 1) * 8;
+    float v[8];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) y[p * 16 + c] = __float2bfloat16_rn(c < cin ? x[p * cin + c] : 0.f);
+    for (int c = 0; c < 8; ++c) v[c] = c0 + c < cin ? x[p * cin + c0 + c] : 0.f;
+    reinterpret_cast<uint4 *>(y)[i] = pack8(v);
 }
 
 // weighted MSE: loss += sum m (y - t)^2 * scale; dz[p][c] = 2 m (y - t) scale
-// (c < 3; channels 3..dzc-1 zero), scale = 1 / (3 sum m)
-__global__ void k_loss(const float *y, const float *t, const float *m, long long P, float scale, bf16 *dz, int dzc,
-                       double *loss) {
-    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// (c < 3; channels 3 .. 31 zero), scale = 1 / (3 sum m).  Four threads per
+// pixel, each writing 8 of dz's 32 channels (16 bytes), the first computing;
+// one atomic per block of a grid of at most kLossBlocks (atomics on the one
+// FP64 sum take about 7 ns each).  128 x 256, batch 8: 56 us with a pixel's 32
+// channels written one by one and an atomic per warp, 28 with one per 64
+// pixels.
+constexpr unsigned kLossBlocks = 608;
+__global__ void __launch_bounds__(256) k_loss(const float *y, const float *t, const float *m, long long P, float scale,
+                                              bf16 *dz, double *loss) {
+    __shared__ double sh[8];
     double l = 0.0;
-    if (p < P) {
-        const float w = m[p];
+    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < 4 * P; i += (long long)gridDim.x * 256) {
+        const long long p = i >> 2;
+        float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if ((i & 3) == 0) {
+            const float w = m[p];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float d = y[p * 3 + c] - t[p * 3 + c];
-            l += (double)(w * d * d) * scale;
-            dz[p * dzc + c] = __float2bfloat16_rn(2.f * w * d * scale);
+            for (int c = 0; c < 3; ++c) {
+                const float d = y[p * 3 + c] - t[p * 3 + c];
+                l += (double)(w * d * d) * scale;
+                v[c] = 2.f * w * d * scale;
+            }
         }
-        for (int c = 3; c < dzc; ++c) dz[p * dzc + c] = __float2bfloat16_rn(0.f);
+        reinterpret_cast<uint4 *>(dz)[i] = pack8(v);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = l;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) l += sh[w];
+        atomicAdd(loss, l);
+    }
 }
 
-// Adam on the FP32 master parameters (Kingma & Ba, bias-corrected)
-__global__ void k_adam(float *p, float *m, float *v, const float *g, long long n, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+// All layers' parameters in one launch: Adam on the FP32 masters (Kingma & Ba,
+// bias-corrected; step = 0 leaves them as they are) and the BF16 copies the
+// convolutions read, w[co][tap][ci] and wt[ci][8 - tap][co].  A block takes a
+// 32 x 32 tile (co, ci) of one tap, which goes through shared memory so that
+// both copies are written along their rows; behind the tiles, one block per
+// layer takes its biases.  (Adam and a launch per layer with wt written 2
+// bytes at a time: 90 us in all; now 23.)
+constexpr int kLayersMax = 18;
+struct PackLayer {
+    long long woff, boff;      // offsets in the master buffer
+    bf16 *w, *wt;
+    int cout, cin, tile0;      // padded channels; the layer's first block
+};
+struct PackArgs {
+    PackLayer L[kLayersMax];
+    int n, tiles;              // layers, weight tiles of all of them
+    float *p, *m, *v;
+    const float *g;
+    int step;
+    float lr, b1, b2, eps, c1, c2;
+};
+__device__ __forceinline__ float adam_step(const PackArgs &a, long long i) {
+    if (!a.step) return a.p[i];
+    const float gi = a.g[i];
+    const float mi = a.b1 * a.m[i] + (1.f - a.b1) * gi;
+    const float vi = a.b2 * a.v[i] + (1.f - a.b2) * gi * gi;
+    a.m[i] = mi;
+    a.v[i] = vi;
+    const float pn = a.p[i] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+    a.p[i] = pn;
+    return pn;
 }
-
-// BF16 copies of one layer: w[co][tap][ci] and wt[ci][8 - tap][co]
-__global__ void k_pack_weights(const float *wf, bf16 *w, bf16 *wt, int coutp, int cinp) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long n = (long long)coutp * 9 * cinp;
-    if (i >= n) return;
-    const int ci = (int)(i % cinp);
-    const int tap = (int)((i / cinp) % 9);
-    const int co = (int)(i / (9LL * cinp));
-    const bf16 v = __float2bfloat16_rn(wf[i]);
-    w[i] = v;
-    wt[((long long)ci * 9 + (8 - tap)) * coutp + co] = v;
+__global__ void __launch_bounds__(256) k_adam_pack(const __grid_constant__ PackArgs a) {
+    __shared__ float tile[32][33];
+    const int b = blockIdx.x;
+    if (b >= a.tiles) {
+        const PackLayer &l = a.L[b - a.tiles];
+        if ((int)threadIdx.x < l.cout) adam_step(a, l.boff + threadIdx.x);
+        return;
+    }
+    int k = 0;
+    while (k + 1 < a.n && b >= a.L[k + 1].tile0) ++k;
+    const PackLayer &l = a.L[k];
+    const int nci = (l.cin + 31) / 32, r = b - l.tile0, tap = r % 9, q = r / 9;
+    const int ci0 = (q % nci) * 32, co0 = (q / nci) * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int j = 0; j < 32; j += 8) {
+        const int co = co0 + ty + j, ci = ci0 + tx;
+        if (ci < l.cin) {
+            const long long i = ((long long)co * 9 + tap) * l.cin + ci;
+            const float v = adam_step(a, l.woff + i);
+            tile[ty + j][tx] = v;
+            l.w[i] = __float2bfloat16_rn(v);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 32; j += 8) {
+        const int ci = ci0 + ty + j, co = co0 + tx;
+        if (ci < l.cin) l.wt[((long long)ci * 9 + (8 - tap)) * l.cout + co] = __float2bfloat16_rn(tile[tx][ty + j]);
+    }
 }
 
 }  // namespace unet
@@ -1614,7 +1722,7 @@ bool launch_col(lbm_unet *u, const ConvArgs &a, lbm_status *st) {
     c.HB = H <= 128 ? H : 128;
     c.NB = std::max(1, 128 / c.HB);
     c.ytiles = (H + c.HB - 1) / c.HB;
-    const int groups = c.ytiles * ((N + c.NB - 1) / c.NB), nblocks = a.cout / NT;
+    const int groups = c.ytiles * ((N + c.NB - 1) / c.NB), nblocks = (a.cout + NT - 1) / NT;
     const long long tiles = (long long)groups * W * nblocks;
     c.L = (int)std::min<long long>(W, (tiles + u->sms - 1) / u->sms);
     c.runs = (W + c.L - 1) / c.L;
@@ -1644,8 +1752,10 @@ bool launch_col(lbm_unet *u, const ConvArgs &a, lbm_status *st) {
     const cuuint64_t gdB[2] = {(cuuint64_t)9 * a.cin, (cuuint64_t)a.wrows};
     const cuuint64_t gsB[1] = {(cuuint64_t)9 * a.cin * 2};
     const cuuint32_t boxB[2] = {(cuuint32_t)BK, (cuuint32_t)NT};
-    if (!image(&ta, a.x + a.xo, a.cin, a.xc, BK, c.HB + 2) || !image(&ty, a.y + a.yo, a.cout, a.yc, NT, c.HB) ||
-        !image(&tg, a.gate ? a.gate + a.go : a.y + a.yo, a.cout, a.gate ? a.gc : a.yc, NT, c.HB) ||
+    // (maps the kernel does not use stand for the input)
+    if (!image(&ta, a.x + a.xo, a.cin, a.xc, BK, c.HB + 2) ||
+        !(a.yf ? image(&ty, a.x + a.xo, a.cin, a.xc, BK, c.HB) : image(&ty, a.y + a.yo, a.cout, a.yc, NT, c.HB)) ||
+        !(a.gate ? image(&tg, a.gate + a.go, a.cout, a.gc, NT, c.HB) : image(&tg, a.x + a.xo, a.cin, a.xc, BK, c.HB)) ||
         enc(&tb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void *)a.w, gdB, gsB, boxB, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
             swz(BK), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
@@ -1669,7 +1779,9 @@ bool launch_col(lbm_unet *u, const ConvArgs &a, lbm_status *st) {
 
 bool conv_col(lbm_unet *u, const ConvArgs &a, lbm_status *st) {
     auto al = [](const void *p) { return (uintptr_t)p % 16 == 0; };
-    if (a.cin > 128 || a.xc % 8 || a.xo % 8 || a.yc % 8 || a.yo % 8 || !al(a.x) || !al(a.w) || !al(a.y) || !a.y ||
+    // an FP32 output (the head) has up to 4 channels and weights padded to 32 rows
+    if (a.cin > 128 || a.xc % 8 || a.xo % 8 || a.yc % 8 || a.yo % 8 || !al(a.x) || !al(a.w) || !al(a.y) ||
+        (a.yf ? (a.yfc > 4 || a.wrows != 32 || a.relu || a.gate || a.cin != 32) : !a.y) ||
         (a.gate && (a.gc % 8 || a.go % 8 || !al(a.gate))))
         return false;
     if (a.cin == 128) {
@@ -1679,7 +1791,7 @@ bool conv_col(lbm_unet *u, const ConvArgs &a, lbm_status *st) {
         if (a.cout == 32) return launch_col<64, 32, 1, true>(u, a, st);
     } else if (a.cin == 32) {
         if (a.cout % 64 == 0) return launch_col<32, 64, 1, true>(u, a, st);
-        if (a.cout == 32) return launch_col<32, 32, 1, true>(u, a, st);
+        if (a.cout == 32 || a.yf) return launch_col<32, 32, 1, true>(u, a, st);
     } else if (a.cin == 16) {
         if (a.cout == 32) return launch_col<16, 32, 1, true>(u, a, st);
     }
@@ -1741,6 +1853,8 @@ lbm_status conv(lbm_unet *u, int li, const bf16 *x, int xc, int xo, int n, int H
     }
     const long long M = (long long)n * H * W;
     if (!yf && a.cout % 16 == 0 && a.cin % 16 == 0) return conv_tc(u, a, M);
+    lbm_status st = LBM_OK;
+    if (yf && conv_col(u, a, &st)) return st;
     dim3 grid(nblk(M, CBM), nblk(a.cout, CBN));
     if (a.cin % 32 == 0) k_conv<32><<<grid, 256, 0, u->stream>>>(a);
     else k_conv<16><<<grid, 256, 0, u->stream>>>(a);
@@ -1869,34 +1983,52 @@ lbm_status wgrad(lbm_unet *u, int li, const bf16 *dz, int dzc, const bf16 *x, in
     return bias_grad(u, dz, dzc, l.cout, P, u->g + l.boff);
 }
 
-lbm_status repack(lbm_unet *u) {
+// the BF16 copies from the masters, after an Adam step with these factors (null: none)
+lbm_status adam_pack(lbm_unet *u, const float *lr_b1_b2_eps) {
+    PackArgs a{};
+    a.n = kL;
     for (int i = 0; i < kL; ++i) {
         const Layer &l = u->L[i];
-        const long long n = (long long)l.coutp * 9 * l.cinp;
-        k_pack_weights<<<nblk(n, 256), 256, 0, u->stream>>>(u->p + l.woff, l.w, l.wt, l.coutp, l.cinp);
-        U_CUDA(u, cudaGetLastError());
+        a.L[i] = PackLayer{(long long)l.woff, (long long)l.boff, l.w, l.wt, l.coutp, l.cinp, a.tiles};
+        a.tiles += 9 * (l.coutp / 32) * ((l.cinp + 31) / 32);
     }
+    a.p = u->p;
+    a.m = u->m;
+    a.v = u->v;
+    a.g = u->g;
+    if (lr_b1_b2_eps) {
+        a.step = 1;
+        a.lr = lr_b1_b2_eps[0];
+        a.b1 = lr_b1_b2_eps[1];
+        a.b2 = lr_b1_b2_eps[2];
+        a.eps = lr_b1_b2_eps[3];
+        a.c1 = 1.f - powf(a.b1, (float)u->adam_t);
+        a.c2 = 1.f - powf(a.b2, (float)u->adam_t);
+    }
+    k_adam_pack<<<a.tiles + a.n, 256, 0, u->stream>>>(a);
+    U_CUDA(u, cudaGetLastError());
     return LBM_OK;
 }
 
-lbm_status forward(lbm_unet *u, const float *xin, int n) {
+// the prediction goes to yout
+lbm_status forward(lbm_unet *u, const float *xin, int n, float *yout) {
     const int H = u->H, W = u->W;
     const int H2 = H / 2, W2 = W / 2, H4 = H / 4, W4 = W / 4, H8 = H / 8, W8 = W / 8;
     lbm_status st;
     const long long P = (long long)n * H * W;
-    k_pack_input<<<nblk(P, 256), 256, 0, u->stream>>>(xin, u->cin, u->x0, P);
+    k_pack_input<<<nblk(2 * P, 256), 256, 0, u->stream>>>(xin, u->cin, u->x0, P);
     U_CUDA(u, cudaGetLastError());
 #define FW(li, x, xc, xo, h, w, y, yc, yo) \
     if ((st = conv(u, li, x, xc, xo, n, h, w, y, yc, yo, true)) != LBM_OK) return st;
     FW(E1A, u->x0, 16, 0, H, W, u->e1a, 32, 0);
     FW(E1B, u->e1a, 32, 0, H, W, u->cat1, 64, 32);
-    k_pool<<<nblk((long long)n * H2 * W2 * 32, 256), 256, 0, u->stream>>>(u->cat1, 64, 32, u->p1, 32, 0, n, H, W, 32);
+    k_pool<<<dim3(nblk(W2 * 32 / 8, 256), n * H2), 256, 0, u->stream>>>(u->cat1, 64, 32, u->p1, 32, 0, H, W, 32);
     FW(E2A, u->p1, 32, 0, H2, W2, u->e2a, 64, 0);
     FW(E2B, u->e2a, 64, 0, H2, W2, u->cat2, 128, 64);
-    k_pool<<<nblk((long long)n * H4 * W4 * 64, 256), 256, 0, u->stream>>>(u->cat2, 128, 64, u->p2, 64, 0, n, H2, W2, 64);
+    k_pool<<<dim3(nblk(W4 * 64 / 8, 256), n * H4), 256, 0, u->stream>>>(u->cat2, 128, 64, u->p2, 64, 0, H2, W2, 64);
     FW(E3A, u->p2, 64, 0, H4, W4, u->e3a, 128, 0);
     FW(E3B, u->e3a, 128, 0, H4, W4, u->cat3, 256, 128);
-    k_pool<<<nblk((long long)n * H8 * W8 * 128, 256), 256, 0, u->stream>>>(u->cat3, 256, 128, u->p3, 128, 0, n, H4, W4, 128);
+    k_pool<<<dim3(nblk(W8 * 128 / 8, 256), n * H8), 256, 0, u->stream>>>(u->cat3, 256, 128, u->p3, 128, 0, H4, W4, 128);
     FW(BA, u->p3, 128, 0, H8, W8, u->ba, 256, 0);
     FW(BB, u->ba, 256, 0, H8, W8, u->bb, 256, 0);
     k_up<<<dim3(nblk((long long)W4 * 256 / 8, 256), n * H4), 256, 0, u->stream>>>(u->bb, 256, 0, u->u3in, 256, 0, n, H4, W4, 256);
@@ -1912,7 +2044,7 @@ lbm_status forward(lbm_unet *u, const float *xin, int n) {
     FW(D1A, u->cat1, 64, 0, H, W, u->d1a, 32, 0);
     FW(D1B, u->d1a, 32, 0, H, W, u->d1, 32, 0);
 #undef FW
-    if ((st = conv(u, HEAD, u->d1, 32, 0, n, H, W, nullptr, 0, 0, true, nullptr, 0, 0, u->yf, 3)) != LBM_OK) return st;
+    if ((st = conv(u, HEAD, u->d1, 32, 0, n, H, W, nullptr, 0, 0, true, nullptr, 0, 0, yout, 3)) != LBM_OK) return st;
     U_CUDA(u, cudaGetLastError());
     return LBM_OK;
 }
@@ -1925,7 +2057,7 @@ lbm_status backward(lbm_unet *u, const float *t, const float *m, int n, float sc
     lbm_status st;
     U_CUDA(u, cudaMemsetAsync(u->g, 0, u->nparam * sizeof(float), u->stream));
     U_CUDA(u, cudaMemsetAsync(u->loss, 0, sizeof(double), u->stream));
-    k_loss<<<nblk(P, 256), 256, 0, u->stream>>>(u->yf, t, m, P, scale, u->g_head, 32, u->loss);
+    k_loss<<<std::min(nblk(4 * P, 256), kLossBlocks), 256, 0, u->stream>>>(u->yf, t, m, P, scale, u->g_head, u->loss);
     U_CUDA(u, cudaGetLastError());
 #define WG(li, dz, dzc, x, xc, xo, h, w) \
     if ((st = wgrad(u, li, dz, dzc, x, xc, xo, n, h, w)) != LBM_OK) return st;
@@ -1940,8 +2072,7 @@ lbm_status backward(lbm_unet *u, const float *t, const float *m, int n, float sc
     DG(D1A, u->g_d1a, 32, H, W, u->g_cat1, 64, 0, u->cat1, 64, 0);  // [dz up1 | dz enc1b (decoder part)]
     WG(U1, u->g_cat1, 64, u->u1in, 64, 0, H, W);
     DG(U1, u->g_cat1, 64, H, W, u->g_u1in, 64, 0, nullptr, 0, 0);
-    k_up_back<<<nblk((long long)n * H2 * W2 * 64, 256), 256, 0, u->stream>>>(u->g_u1in, 64, 0, u->d2, 64, 0, u->g_d2, 64, 0,
-                                                                            n, H2, W2, 64);
+    k_up_back<<<dim3(nblk(W2 * 64 / 8, 256), n * H2), 256, 0, u->stream>>>(u->g_u1in, 64, 0, u->d2, 64, 0, u->g_d2, 64, 0, H2, W2, 64);
     // decoder level 2
     WG(D2B, u->g_d2, 64, u->d2a, 64, 0, H2, W2);
     DG(D2B, u->g_d2, 64, H2, W2, u->g_d2a, 64, 0, u->d2a, 64, 0);
@@ -1949,8 +2080,8 @@ lbm_status backward(lbm_unet *u, const float *t, const float *m, int n, float sc
     DG(D2A, u->g_d2a, 64, H2, W2, u->g_cat2, 128, 0, u->cat2, 128, 0);
     WG(U2, u->g_cat2, 128, u->u2in, 128, 0, H2, W2);
     DG(U2, u->g_cat2, 128, H2, W2, u->g_u2in, 128, 0, nullptr, 0, 0);
-    k_up_back<<<nblk((long long)n * H4 * W4 * 128, 256), 256, 0, u->stream>>>(u->g_u2in, 128, 0, u->d3, 128, 0, u->g_d3,
-                                                                             128, 0, n, H4, W4, 128);
+    k_up_back<<<dim3(nblk(W4 * 128 / 8, 256), n * H4), 256, 0, u->stream>>>(u->g_u2in, 128, 0, u->d3, 128, 0, u->g_d3,
+                                                                             128, 0, H4, W4, 128);
     // decoder level 3
     WG(D3B, u->g_d3, 128, u->d3a, 128, 0, H4, W4);
     DG(D3B, u->g_d3, 128, H4, W4, u->g_d3a, 128, 0, u->d3a, 128, 0);
@@ -1958,28 +2089,28 @@ lbm_status backward(lbm_unet *u, const float *t, const float *m, int n, float sc
     DG(D3A, u->g_d3a, 128, H4, W4, u->g_cat3, 256, 0, u->cat3, 256, 0);
     WG(U3, u->g_cat3, 256, u->u3in, 256, 0, H4, W4);
     DG(U3, u->g_cat3, 256, H4, W4, u->g_u3in, 256, 0, nullptr, 0, 0);
-    k_up_back<<<nblk((long long)n * H8 * W8 * 256, 256), 256, 0, u->stream>>>(u->g_u3in, 256, 0, u->bb, 256, 0, u->g_bb,
-                                                                             256, 0, n, H8, W8, 256);
+    k_up_back<<<dim3(nblk(W8 * 256 / 8, 256), n * H8), 256, 0, u->stream>>>(u->g_u3in, 256, 0, u->bb, 256, 0, u->g_bb,
+                                                                             256, 0, H8, W8, 256);
     // bottleneck
     WG(BB, u->g_bb, 256, u->ba, 256, 0, H8, W8);
     DG(BB, u->g_bb, 256, H8, W8, u->g_ba, 256, 0, u->ba, 256, 0);
     WG(BA, u->g_ba, 256, u->p3, 128, 0, H8, W8);
     DG(BA, u->g_ba, 256, H8, W8, u->g_p3, 128, 0, nullptr, 0, 0);
     // encoder level 3: dz of enc3b = decoder part + pooling path (gated by enc3b > 0)
-    k_pool_back<<<nblk((long long)n * H4 * W4 * 128, 256), 256, 0, u->stream>>>(u->g_p3, 128, 0, u->cat3, 256, 128,
-                                                                               u->g_cat3, 256, 128, n, H4, W4, 128, 1);
+    k_pool_back<<<dim3(nblk(W4 * 128 / 8, 256), n * H4), 256, 0, u->stream>>>(u->g_p3, 128, 0, u->cat3, 256, 128,
+                                                                               u->g_cat3, 256, 128, H4, W4, 128);
     WG(E3B, u->g_cat3 + 128, 256, u->e3a, 128, 0, H4, W4);
     DG(E3B, u->g_cat3 + 128, 256, H4, W4, u->g_e3a, 128, 0, u->e3a, 128, 0);
     WG(E3A, u->g_e3a, 128, u->p2, 64, 0, H4, W4);
     DG(E3A, u->g_e3a, 128, H4, W4, u->g_p2, 64, 0, nullptr, 0, 0);
-    k_pool_back<<<nblk((long long)n * H2 * W2 * 64, 256), 256, 0, u->stream>>>(u->g_p2, 64, 0, u->cat2, 128, 64, u->g_cat2,
-                                                                              128, 64, n, H2, W2, 64, 1);
+    k_pool_back<<<dim3(nblk(W2 * 64 / 8, 256), n * H2), 256, 0, u->stream>>>(u->g_p2, 64, 0, u->cat2, 128, 64, u->g_cat2,
+                                                                              128, 64, H2, W2, 64);
     WG(E2B, u->g_cat2 + 64, 128, u->e2a, 64, 0, H2, W2);
     DG(E2B, u->g_cat2 + 64, 128, H2, W2, u->g_e2a, 64, 0, u->e2a, 64, 0);
     WG(E2A, u->g_e2a, 64, u->p1, 32, 0, H2, W2);
     DG(E2A, u->g_e2a, 64, H2, W2, u->g_p1, 32, 0, nullptr, 0, 0);
-    k_pool_back<<<nblk((long long)n * H * W * 32, 256), 256, 0, u->stream>>>(u->g_p1, 32, 0, u->cat1, 64, 32, u->g_cat1, 64,
-                                                                            32, n, H, W, 32, 1);
+    k_pool_back<<<dim3(nblk(W * 32 / 8, 256), n * H), 256, 0, u->stream>>>(u->g_p1, 32, 0, u->cat1, 64, 32, u->g_cat1, 64,
+                                                                            32, H, W, 32);
     WG(E1B, u->g_cat1 + 32, 64, u->e1a, 32, 0, H, W);
     DG(E1B, u->g_cat1 + 32, 64, H, W, u->g_e1a, 32, 0, u->e1a, 32, 0);
     WG(E1A, u->g_e1a, 32, u->x0, 16, 0, H, W);
@@ -2113,7 +2244,7 @@ lbm_status lbm_unet_set_params(lbm_unet *u, const float *host) {
     U_CUDA(u, cudaMemsetAsync(u->m, 0, u->nparam * 4, u->stream));
     U_CUDA(u, cudaMemsetAsync(u->v, 0, u->nparam * 4, u->stream));
     u->adam_t = 0;
-    lbm_status st = repack(u);
+    lbm_status st = adam_pack(u, nullptr);
     if (st != LBM_OK) return st;
     U_CUDA(u, cudaStreamSynchronize(u->stream));
     return LBM_OK;
@@ -2155,17 +2286,14 @@ lbm_status lbm_unet_get_params(lbm_unet *u, float *host) {
 lbm_status lbm_unet_forward(lbm_unet *u, const float *x_dev, float *y_dev, int n) {
     if (!u || !x_dev || !y_dev) return ufail(u, LBM_ERR_ARG, "NULL argument");
     if (n < 1 || n > u->B) return ufail(u, LBM_ERR_ARG, "batch size out of range");
-    lbm_status st = forward(u, x_dev, n);
-    if (st != LBM_OK) return st;
-    U_CUDA(u, cudaMemcpyAsync(y_dev, u->yf, (size_t)n * u->H * u->W * 3 * 4, cudaMemcpyDeviceToDevice, u->stream));
-    return LBM_OK;
+    return forward(u, x_dev, n, y_dev);
 }
 
 lbm_status lbm_unet_grad(lbm_unet *u, const float *x_dev, const float *t_dev, const float *m_dev, int n, float scale,
                          double *loss_host, float *grad_host) {
     if (!u || !x_dev || !t_dev || !m_dev) return ufail(u, LBM_ERR_ARG, "NULL argument");
     if (n < 1 || n > u->B) return ufail(u, LBM_ERR_ARG, "batch size out of range");
-    lbm_status st = forward(u, x_dev, n);
+    lbm_status st = forward(u, x_dev, n, u->yf);
     if (st == LBM_OK) st = backward(u, t_dev, m_dev, n, scale);
     if (st != LBM_OK) return st;
     if ((st = check_tc(u)) != LBM_OK) return st;
@@ -2180,18 +2308,15 @@ lbm_status lbm_unet_grad(lbm_unet *u, const float *x_dev, const float *t_dev, co
 lbm_status lbm_unet_adam(lbm_unet *u, float lr, float beta1, float beta2, float eps) {
     if (!u) return ufail(nullptr, LBM_ERR_ARG, "NULL argument");
     u->adam_t += 1;
-    const float c1 = 1.f - powf(beta1, (float)u->adam_t), c2 = 1.f - powf(beta2, (float)u->adam_t);
-    k_adam<<<nblk((long long)u->nparam, 256), 256, 0, u->stream>>>(u->p, u->m, u->v, u->g, (long long)u->nparam, lr,
-                                                                   beta1, beta2, eps, c1, c2);
-    U_CUDA(u, cudaGetLastError());
-    return repack(u);
+    const float f[4] = {lr, beta1, beta2, eps};
+    return adam_pack(u, f);
 }
 
 lbm_status lbm_unet_train_step(lbm_unet *u, const float *x_dev, const float *t_dev, const float *m_dev, int n,
                                float scale, float lr, double *loss_dev) {
     if (!u || !x_dev || !t_dev || !m_dev) return ufail(u, LBM_ERR_ARG, "NULL argument");
     if (n < 1 || n > u->B) return ufail(u, LBM_ERR_ARG, "batch size out of range");
-    lbm_status st = forward(u, x_dev, n);
+    lbm_status st = forward(u, x_dev, n, u->yf);
     if (st == LBM_OK) st = backward(u, t_dev, m_dev, n, scale);
     if (st == LBM_OK) st = lbm_unet_adam(u, lr, 0.9f, 0.999f, 1e-8f);
     if (st != LBM_OK) return st;
