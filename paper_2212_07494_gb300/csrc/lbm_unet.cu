@@ -586,6 +586,42 @@ __global__ void __launch_bounds__(160) k_conv_tma(const ConvArgs a, const __grid
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NCOL));
 }
 
+// --------------------------------------------- issuing copies and MMAs cheaply
+__device__ __forceinline__ void mbar_init(unsigned long long *m, int count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(m)), "r"(count));
+}
+__device__ __forceinline__ void mbar_expect(unsigned long long *m, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(m)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned long long *m) {
+    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(m)) : "memory");
+}
+// One thread of a converged warp issues an MMA: accumulator acc (added to when
+// `more`), low and high words of the A and B descriptors.  The
+// operands are computed from kernel parameters and block indices alone and no
+// wait's result steers the loop, so that they can stay in uniform registers,
+// which the instruction reads (a single lane issuing out of a diverged warp
+// took 120 - 150 clocks).
+__device__ __forceinline__ void mma_elect(unsigned acc, unsigned alo, unsigned blo, unsigned ahi, unsigned bhi, uint32_t idesc,
+                                          unsigned more) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %3};\n\t"
+        "mov.b64 db, {%2, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t"
+        "}\n" ::"r"(acc),
+        "r"(alo), "r"(blo), "r"(ahi), "r"(bhi), "r"(idesc), "r"(more));
+}
+__device__ __forceinline__ void commit_elect(unsigned mbar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t"
+        "}\n" ::"r"(mbar));
+}
+
 // ------------------------------------------------------------ weight gradient
 struct WgradArgs {
     const bf16 *dz;
@@ -693,26 +729,36 @@ __global__ void __launch_bounds__(128) k_wgrad(const WgradArgs a) {
 // 5th-generation tensor cores, D[m][co] += sum_p A[m][p] B[co][p]: a row m of
 // D is one input channel of one (tap, channel block) pair, 128 rows per CTA
 // (128 / CA pairs of CA channels), and N = the layer's padded output
-// channels.  The contraction runs over pixels in blocks of 64 along one x
-// column: HB rows y of NB images (HB NB = 64), as the forward kernel's column
+// channels.  The contraction runs over pixels in blocks of 128 along one x
+// column: HB rows y of NB images (HB NB = 128), as the forward kernel's column
 // tiles.  The x operand of pair (tap, block) for a pixel block is the TMA box
 // at column x + dx (modulo W, or reading zeros outside the image) and rows
 // y + dy (zeros outside), the dz operand the unshifted box, so every operand
-// is one plain 4-D box per atom.
+// is one plain 4-D box per atom; rows past the image's end and images past the
+// batch's are zeros in both.
 // Both operands arrive channel-contiguous, i.e. MN-major: an atom is CA (A)
 // or CB (B) channels wide -- the swizzle width, 64 -> 128 B, 32 -> 64 B,
-// 16 -> 32 B -- and 64 pixel rows deep; the atoms of an operand lie one atom
+// 16 -> 32 B -- and 128 pixel rows deep; the atoms of an operand lie one atom
 // apart (the descriptor's leading offset), 8-row pixel groups 8 rows apart
 // (its stride offset), and the MMA's K slices of 16 pixels start 16 rows
 // apart.  The instruction descriptor marks both operands MN-major.  CTAs
 // split the pixel blocks between them and add their 128 x N partial sums to
-// dW with FP32 atomics.  One thread issues the copies, one the MMAs; four
-// stages; every wait is bounded, as in k_conv_tma.
+// dW with FP32 atomics.
+// What bounds it is issuing: a barrier round costs about 350 clocks, a copy
+// 60 - 100 and an MMA 110.  So a block is 128 pixels (64 took twice the
+// copies), every copy of a stage is issued by a lane of its own, whose
+// coordinates are computed once, and the MMA warp stays converged.  us a
+// launch before and after (one issuing thread, 64 pixels; 128 x 256, batch 8,
+// cold cache): 32 -> 32 channels at full resolution 54 and 23, 64 -> 64 at half
+// 46 and 14, 256 -> 256 at an eighth 45 and 14.  Every wait is bounded; after a
+// failed one the loops run on without waiting.
 struct WgTcArgs {
     float *dw;           // [cout][9][cin]
     int cin, cout;       // padded channels (cout = the MMA's N)
     int H, W;
-    int HB, NB;          // a pixel block: HB rows of NB images at one x
+    int HB, NB;          // a pixel block: HB rows of NB images at one x (HB NB = 128)
+    int ytiles;          // pixel blocks per column of an image
+    int S;               // stages
     int wrapx;
     int CA, CB;          // atom widths of the x and dz operands (channels)
     int pairs;           // 9 cin / CA (tap, channel block) pairs
@@ -720,9 +766,10 @@ struct WgTcArgs {
     int kb_per;          // pixel blocks per CTA
     unsigned ncol;       // TMEM columns (power of two >= 32, >= cout)
 };
-constexpr int WG_S = 4;
-constexpr unsigned WG_ABYTES = 128 * 64 * 2;  // the x operand: 128 rows of 64 pixels
-constexpr unsigned wg_stage_bytes(int cout) { return WG_ABYTES + (unsigned)cout * 64 * 2; }
+constexpr int WG_SMAX = 4;
+constexpr int WG_K = 128;                        // pixels per block
+constexpr unsigned WG_ABYTES = 128 * WG_K * 2;   // the x operand: 128 rows
+constexpr unsigned wg_stage_bytes(int cout) { return WG_ABYTES + (unsigned)cout * WG_K * 2; }
 
 __device__ __forceinline__ uint64_t sw_mode_bytes(int rowbytes) { return rowbytes == 128 ? 2 : (rowbytes == 64 ? 4 : 6); }
 
@@ -748,31 +795,30 @@ __device__ __forceinline__ void tma_load4(unsigned dst, const CUtensorMap *map, 
 __global__ void __launch_bounds__(160) k_wgrad_tc(const WgTcArgs a, const __grid_constant__ CUtensorMap tmX,
                                                   const __grid_constant__ CUtensorMap tmZ, int *err) {
     extern __shared__ __align__(1024) unsigned char wg_smem[];
-    __shared__ __align__(8) unsigned long long full[WG_S], empty[WG_S], done;
+    __shared__ __align__(8) unsigned long long full[WG_SMAX], empty[WG_SMAX], done;
     __shared__ unsigned tmem_base;
     __shared__ volatile int s_fail;
-    __shared__ int s_consumed;
+    __shared__ int s_issued;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     unsigned char *sm = (unsigned char *)(((uintptr_t)wg_smem + 1023) & ~(uintptr_t)1023);
-    const unsigned STAGE = wg_stage_bytes(a.cout);
+    const unsigned STAGE = wg_stage_bytes(a.cout), base = smem_addr(sm);
     const int per_tile = 128 / a.CA;                // pairs per CTA
     const int p0 = blockIdx.y * per_tile;
     const int np = min(per_tile, a.pairs - p0);     // pairs this CTA loads (>= 1)
     const int cblocks = a.cin / a.CA;
-    const int ytiles = a.H / a.HB;
     const int nb_atoms = a.cout / a.CB;
-    const unsigned arow = 2u * a.CA, brow = 2u * a.CB;      // bytes of one pixel row of an atom
-    const unsigned aatom = 64u * arow, batom = 64u * brow;  // bytes of one atom
+    const unsigned arow = 2u * a.CA, brow = 2u * a.CB;          // bytes of one pixel row of an atom
+    const unsigned aatom = WG_K * arow, batom = WG_K * brow;    // bytes of one atom
     const long long kb0 = (long long)blockIdx.x * a.kb_per;
     const int KB = (int)min((long long)a.kb_per, a.kb_total - kb0);  // >= 1
     if (tid == 0) {
         s_fail = 0;
-        s_consumed = 0;
-        for (int s = 0; s < WG_S; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&full[s])), "r"(1));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&empty[s])), "r"(1));
+        s_issued = 0;
+        for (int s = 0; s < a.S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(&done)), "r"(1));
+        mbar_init(&done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (warp == 0) {
@@ -784,58 +830,65 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(const WgTcArgs a, const __grid
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const unsigned tmem = tmem_base;
-    int issued = 0;
-    if (tid == 0) {
-        // ---- producer: np x boxes and nb_atoms dz boxes per pixel block
+    if (warp == 0) {
+        // ---- producer: lane j < np loads pair j's x box, the next nb_atoms
+        // lanes the dz boxes (np + nb_atoms <= 12)
         const unsigned tx = (unsigned)np * aatom + (unsigned)nb_atoms * batom;
+        const bool isx = lane < np, loads = lane < np + nb_atoms;
+        const int pr = p0 + lane, tap = pr / cblocks, j = lane - np;
+        const int dy = isx ? tap / 3 - 1 : 0, dx = isx ? tap % 3 - 1 : 0;
+        const int c0 = isx ? (pr - tap * cblocks) * a.CA : j * a.CB;
+        const unsigned off = isx ? lane * aatom : WG_ABYTES + j * batom;
+        const CUtensorMap *map = isx ? &tmX : &tmZ;
+        int xcol = (int)(kb0 % a.W), yt = (int)(kb0 / a.W % a.ytiles), ng = (int)(kb0 / a.W / a.ytiles);
+        int s = 0, ph = 1;
         for (int i = 0; i < KB; ++i) {
-            const int s = i % WG_S;
-            if (i >= WG_S && !ws_wait(&empty[s], (i / WG_S - 1) & 1, &s_fail)) break;
-            const long long kb = kb0 + i;
-            const int xcol = (int)(kb % a.W);
-            const long long rest = kb / a.W;
-            const int y0 = (int)(rest % ytiles) * a.HB, n0 = (int)(rest / ytiles) * a.NB;
-            const unsigned sa = smem_addr(sm + (size_t)s * STAGE), sb = sa + WG_ABYTES, mb = smem_addr(&full[s]);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(tx) : "memory");
-            for (int j = 0; j < np; ++j) {
-                const int pr = p0 + j;
-                const int tap = pr / cblocks, c0 = (pr - tap * cblocks) * a.CA;
-                const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-                int xx = xcol + dx;
-                if (a.wrapx) xx = xx < 0 ? xx + a.W : (xx >= a.W ? xx - a.W : xx);
-                tma_load4(sa + j * aatom, &tmX, c0, xx, y0 + dy, n0, mb);
+            if (lane == 0) {
+                if (i >= a.S) ws_wait(&empty[s], ph, &s_fail);
+                if (!s_fail) {
+                    mbar_expect(&full[s], tx);
+                    s_issued = i + 1;
+                }
             }
-            for (int j = 0; j < nb_atoms; ++j) tma_load4(sb + j * batom, &tmZ, j * a.CB, xcol, y0, n0, mb);
-            issued = i + 1;
+            if (__shfl_sync(0xffffffffu, lane == 0 && s_fail ? 1 : 0, 0)) break;
+            int xx = xcol + dx;
+            if (a.wrapx) xx = xx < 0 ? xx + a.W : (xx >= a.W ? xx - a.W : xx);
+            if (loads) tma_load4(base + s * STAGE + off, map, c0, xx, yt * a.HB + dy, ng * a.NB, smem_addr(&full[s]));
+            __syncwarp();
+            if (++xcol == a.W) {
+                xcol = 0;
+                if (++yt == a.ytiles) {
+                    yt = 0;
+                    ++ng;
+                }
+            }
+            if (++s == a.S) {
+                s = 0;
+                ph ^= 1;
+            }
         }
-    } else if (warp == 4 && lane == 0) {
+    } else if (warp == 4) {
         // ---- MMA issuer: M = 128, N = cout, both operands MN-major
         const uint32_t idesc = tc_idesc(128, a.cout) | (1u << 15) | (1u << 16);
-        const uint64_t amode = sw_mode_bytes(arow), bmode = sw_mode_bytes(brow);
-        int i = 0;
-        for (; i < KB; ++i) {
-            const int s = i % WG_S;
-            if (!ws_wait(&full[s], (i / WG_S) & 1, &s_fail)) break;
+        const uint64_t ad = tc_desc_mn(0, aatom, 8 * arow, sw_mode_bytes(arow)),
+                       bd = tc_desc_mn(0, batom, 8 * brow, sw_mode_bytes(brow));
+        const unsigned ahi = (unsigned)(ad >> 32), bhi = (unsigned)(bd >> 32);
+        const unsigned a16 = (unsigned)ad + (base >> 4), b16 = (unsigned)bd + ((base + WG_ABYTES) >> 4);
+        int s = 0, ph = 0;
+        for (int i = 0; i < KB; ++i) {
+            ws_wait(&full[s], ph, &s_fail);
             asm volatile("tcgen05.fence::after_thread_sync;");
-            const unsigned sa = smem_addr(sm + (size_t)s * STAGE), sb = sa + WG_ABYTES;
+            const unsigned as = a16 + s * (STAGE >> 4), bs = b16 + s * (STAGE >> 4);
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                const uint64_t da = tc_desc_mn(sa + ks * 16 * arow, aatom, 8 * arow, amode);
-                const uint64_t db = tc_desc_mn(sb + ks * 16 * brow, batom, 8 * brow, bmode);
-                const unsigned acc = (i > 0 || ks > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\t"
-                    "setp.ne.b32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t"
-                    "}\n" ::"r"(tmem),
-                    "l"(da), "l"(db), "r"(idesc), "r"(acc));
+            for (int ks = 0; ks < WG_K / 16; ++ks)
+                mma_elect(tmem, as + ks * arow, bs + ks * brow, ahi, bhi, idesc, ks > 0 ? 1u : (unsigned)i);
+            commit_elect(smem_addr(&empty[s]));
+            if (++s == a.S) {
+                s = 0;
+                ph ^= 1;
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_addr(&empty[s])));
         }
-        s_consumed = i;
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-            smem_addr(&done)));
+        commit_elect(smem_addr(&done));
     }
     if (warp < 4) {
         // epilogue: warp w holds rows 32w .. 32w + 31; rows of pairs this CTA
@@ -873,7 +926,7 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(const WgTcArgs a, const __grid
         // copies still in flight land, and issued MMAs finish, before the
         // CTA frees its TMEM and leaves
         volatile int never = 0;
-        for (int i = s_consumed; i < issued; ++i) ws_wait(&full[i % WG_S], (i / WG_S) & 1, &never);
+        for (int i = max(0, s_issued - a.S); i < s_issued; ++i) ws_wait(&full[i % a.S], (i / a.S) & 1, &never);
         ws_wait(&done, 0, &never);
         atomicExch(err, 1);
     }
@@ -919,41 +972,6 @@ struct ColArgs {
 };
 constexpr int COL_WS = 5;         // weight stages when they are streamed
 constexpr int COL_RMAX = 8;
-
-__device__ __forceinline__ void mbar_init(unsigned long long *m, int count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(m)), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect(unsigned long long *m, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(m)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(unsigned long long *m) {
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_addr(m)) : "memory");
-}
-// One thread of a converged warp issues an MMA: accumulator acc (added to when
-// `more`), low words of the A and B descriptors, their common high word.  The
-// operands are computed from kernel parameters and block indices alone and no
-// wait's result steers the loop, so that they can stay in uniform registers,
-// which the instruction reads (a single lane issuing out of a diverged warp
-// took 120 - 150 clocks).
-__device__ __forceinline__ void mma_elect(unsigned acc, unsigned alo, unsigned blo, unsigned hi, uint32_t idesc,
-                                          unsigned more) {
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
-        "mov.b64 da, {%1, %3};\n\t"
-        "mov.b64 db, {%2, %3};\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "elect.sync _|q, 0xffffffff;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t"
-        "}\n" ::"r"(acc),
-        "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(more));
-}
-__device__ __forceinline__ void commit_elect(unsigned mbar) {
-    asm volatile(
-        "{\n\t.reg .pred q;\n\t"
-        "elect.sync _|q, 0xffffffff;\n\t"
-        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t"
-        "}\n" ::"r"(mbar));
-}
 
 template <int BK, int NT, int CB, bool RES>
 __global__ void __launch_bounds__(384) k_conv_col(const ConvArgs a, const __grid_constant__ CUtensorMap tmA,
@@ -1125,7 +1143,7 @@ __global__ void __launch_bounds__(384) k_conv_col(const ConvArgs a, const __grid
                     if (active)
 #pragma unroll
                         for (int ks = 0; ks < BK / 16; ++ks)
-                            mma_elect(acc, a0 + 2 * ks, b0 + 2 * ks, HI, IDESC, ks > 0 ? 1u : (unsigned)(tap + cb));
+                            mma_elect(acc, a0 + 2 * ks, b0 + 2 * ks, HI, HI, IDESC, ks > 0 ? 1u : (unsigned)(tap + cb));
                     if (!RES) {
                         commit_elect(smem_addr(&wempty[ws]));
                         if (++ws == COL_WS) {
@@ -1875,18 +1893,18 @@ lbm_status bias_grad(lbm_unet *u, const bf16 *dz, int dzc, int C, long long P, f
     return LBM_OK;
 }
 
-// The tcgen05 weight gradient when the shape suits its pixel blocks (64
-// pixels of one column: H <= 64 dividing 64 with n a multiple of 64 / H, or H
-// a multiple of 64) and every global address and stride is a multiple of 16
-// bytes.  Returns false (nothing launched) otherwise, and when a tensor map
-// cannot be made.  The pixel blocks are split so that about two CTAs per SM
-// run, each taking at least 8 blocks (its 128 x N atomics stay small against
-// its MMA work).
+// The tcgen05 weight gradient when the shape suits its pixel blocks (H a
+// divisor of 128, or above 128) and every global address and stride is a
+// multiple of 16 bytes.  Returns false (nothing launched) otherwise, and when
+// a tensor map cannot be made.  The pixel blocks are split so that two CTAs
+// per SM run, or one where two stages of it need over half the shared memory,
+// each taking at least 4 blocks (its 128 x N atomics stay small against its
+// MMA work).
 bool launch_wgrad_tc(lbm_unet *u, const Layer &l, const bf16 *dz, int dzc, const bf16 *x, int xc, int xo, int n,
                      int H, int W, lbm_status *st) {
-    const int HB = H <= 64 ? H : 64;
-    const int NB = H <= 64 ? 64 / H : 1;
-    if (H <= 64 ? (64 % H != 0 || n % NB != 0) : (H % 64 != 0)) return false;
+    const int HB = H <= WG_K ? H : WG_K;
+    const int NB = WG_K / HB;
+    if (WG_K % HB != 0) return false;
     const int cin = l.cinp, cout = l.coutp;
     // atom widths are swizzle widths: 16, 32 or 64 channels
     if ((cin < 64 ? (cin != 16 && cin != 32) : cin % 64 != 0) || cout > 256 || (cout < 64 ? cout != 32 : cout % 64 != 0))
@@ -1929,15 +1947,19 @@ bool launch_wgrad_tc(lbm_unet *u, const Layer &l, const bf16 *dz, int dzc, const
     a.CA = CA;
     a.CB = CB;
     a.pairs = 9 * cin / CA;
-    a.kb_total = (long long)n * H * W / 64;
+    a.ytiles = (H + HB - 1) / HB;
+    a.kb_total = (long long)((n + NB - 1) / NB) * a.ytiles * W;
     a.ncol = cout <= 32 ? 32u : (cout <= 64 ? 64u : (cout <= 128 ? 128u : 256u));
     const int mtiles = (a.pairs + 128 / CA - 1) / (128 / CA);
-    long long splits = (2LL * u->sms + mtiles - 1) / mtiles;
-    const long long cap = a.kb_total / 8 > 0 ? a.kb_total / 8 : 1;
+    const size_t stage = wg_stage_bytes(cout), half = 233472 / 2 - 2048;
+    const int ctas = 2 * stage <= half ? 2 : 1;   // per SM
+    a.S = (int)std::min<size_t>(WG_SMAX, (ctas == 2 ? half : (size_t)229376) / stage);
+    long long splits = std::max(1LL, (long long)ctas * u->sms / mtiles);
+    const long long cap = a.kb_total / 4 > 0 ? a.kb_total / 4 : 1;
     if (splits > cap) splits = cap;
     a.kb_per = (int)((a.kb_total + splits - 1) / splits);
     splits = (a.kb_total + a.kb_per - 1) / a.kb_per;  // every CTA gets at least one block
-    const size_t smem = (size_t)WG_S * wg_stage_bytes(256) + 1024;
+    const size_t smem = 229376 + 1024;
     static bool attr = false;
     if (!attr) {
         cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1947,7 +1969,7 @@ bool launch_wgrad_tc(lbm_unet *u, const Layer &l, const bf16 *dz, int dzc, const
         }
         attr = true;
     }
-    const size_t need = (size_t)WG_S * wg_stage_bytes(cout) + 1024;
+    const size_t need = a.S * stage + 1024;
     k_wgrad_tc<<<dim3((unsigned)splits, (unsigned)mtiles), 160, need, u->stream>>>(a, tx, tz, u->tc_err);
     cudaError_t e = cudaGetLastError();
     *st = e == cudaSuccess ? LBM_OK : ufail(u, LBM_ERR_CUDA, std::string("k_wgrad_tc: ") + cudaGetErrorString(e));
