@@ -587,6 +587,11 @@ __global__ void __launch_bounds__(160) k_conv_tma(const ConvArgs a, const __grid
 }
 
 // --------------------------------------------- issuing copies and MMAs cheaply
+// a value all lanes of a converged warp hold, as one the compiler knows to be
+// uniform: the role branches and the MMA operands derived from it can then
+// stay in uniform registers
+__device__ __forceinline__ unsigned uniform(unsigned v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 __device__ __forceinline__ void mbar_init(unsigned long long *m, int count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(m)), "r"(count));
 }
@@ -799,7 +804,7 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(const WgTcArgs a, const __grid
     __shared__ unsigned tmem_base;
     __shared__ volatile int s_fail;
     __shared__ int s_issued;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = (int)uniform(threadIdx.x >> 5), lane = tid & 31;
     unsigned char *sm = (unsigned char *)(((uintptr_t)wg_smem + 1023) & ~(uintptr_t)1023);
     const unsigned STAGE = wg_stage_bytes(a.cout), base = smem_addr(sm);
     const int per_tile = 128 / a.CA;                // pairs per CTA
@@ -829,7 +834,7 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(const WgTcArgs a, const __grid
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    const unsigned tmem = tmem_base;
+    const unsigned tmem = uniform(tmem_base);
     if (warp == 0) {
         // ---- producer: lane j < np loads pair j's x box, the next nb_atoms
         // lanes the dz boxes (np + nb_atoms <= 12)
@@ -992,7 +997,7 @@ __global__ void __launch_bounds__(384) k_conv_col(const ConvArgs a, const __grid
     __shared__ volatile int s_fail;
     __shared__ int s_cols, s_w, s_g;        // columns, weight blocks and gate tiles whose copies were issued
     __shared__ float s_bias[NT];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = (int)uniform(threadIdx.x >> 5), lane = tid & 31;
     unsigned char *sm = (unsigned char *)(((uintptr_t)col_smem + 1023) & ~(uintptr_t)1023);
     const unsigned scol = smem_addr(sm), sw = scol + (unsigned)(c.R * CB * c.colb),
                    so = sw + (RES ? KB : COL_WS) * WB;
@@ -1032,7 +1037,7 @@ __global__ void __launch_bounds__(384) k_conv_col(const ConvArgs a, const __grid
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    const unsigned tmem = tmem_base;
+    const unsigned tmem = uniform(tmem_base);
     // the gate's tile of column i into the output tile that column i will leave from
     auto gate_load = [&](int i) {
         const int k = i >> 1, b = (i & 1) * OB + k % OB;
