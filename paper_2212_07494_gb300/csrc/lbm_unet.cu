@@ -1179,8 +1179,11 @@ __global__ void __launch_bounds__(384) k_conv_col(const ConvArgs a, const __grid
                 p2 ^= 1;
             }
         }
-        // completes when every MMA this warp issued has
+        // completes when every MMA this warp issued has; waited for, so that
+        // no commit's arrival is still on its way to the barriers when the CTA
+        // leaves (the epilogue waits for the accumulators' only)
         commit_elect(smem_addr(&done[me]));
+        ws_wait(&done[me], 0, &s_fail);
     } else {
         // ---- epilogue: group (warp - 4) / 4 takes every second column
         const int grp = (warp - 4) >> 2, q = warp & 3;
