@@ -734,13 +734,14 @@ __global__ void __launch_bounds__(128) k_wgrad(const WgradArgs a) {
 // 5th-generation tensor cores, D[m][co] += sum_p A[m][p] B[co][p]: a row m of
 // D is one input channel of one (tap, channel block) pair, 128 rows per CTA
 // (128 / CA pairs of CA channels), and N = the layer's padded output
-// channels.  The contraction runs over pixels in blocks of 128 along one x
-// column: HB rows y of NB images (HB NB = 128), as the forward kernel's column
+// channels.  The contraction runs over pixels in blocks of 64 along one x
+// column: HB rows y of NB images (HB NB = 64), as the forward kernel's column
 // tiles.  The x operand of pair (tap, block) for a pixel block is the TMA box
 // at column x + dx (modulo W, or reading zeros outside the image) and rows
-// y + dy (zeros outside), the dz operand the unshifted box, so every operand
-// is one plain 4-D box per atom; rows past the image's end and images past the
-// batch's are zeros in both.
+// y + dy (zeros outside), the dz operand the unshifted box.  A stage takes two
+// neighbouring columns, one block after the other, as one 4-D box (channel, y,
+// image, x) per atom; at a periodic edge two boxes, and a row of columns' or
+// the CTA's odd last block goes alone.
 // Both operands arrive channel-contiguous, i.e. MN-major: an atom is CA (A)
 // or CB (B) channels wide -- the swizzle width, 64 -> 128 B, 32 -> 64 B,
 // 16 -> 32 B -- and 128 pixel rows deep; the atoms of an operand lie one atom
@@ -748,9 +749,12 @@ __global__ void __launch_bounds__(128) k_wgrad(const WgradArgs a) {
 // (its stride offset), and the MMA's K slices of 16 pixels start 16 rows
 // apart.  The instruction descriptor marks both operands MN-major.  CTAs
 // split the pixel blocks between them and add their 128 x N partial sums to
-// dW with FP32 atomics.
+// dW with FP32 atomics.  The additions in TMEM truncate, so which pixels one
+// CTA adds, in which order, is part of the result: with longer sums or other
+// members the losses of the next training steps moved by more than two runs
+// differ by themselves.
 // What bounds it is issuing: a barrier round costs about 350 clocks, a copy
-// 60 - 100 and an MMA 110.  So a block is 128 pixels (64 took twice the
+// 60 - 100 and an MMA 110.  So a stage is two blocks (one took twice the
 // copies), every copy of a stage is issued by a lane of its own, whose
 // coordinates are computed once, and the MMA warp stays converged.  us a
 // launch before and after (one issuing thread, 64 pixels; 128 x 256, batch 8,
@@ -761,7 +765,7 @@ struct WgTcArgs {
     float *dw;           // [cout][9][cin]
     int cin, cout;       // padded channels (cout = the MMA's N)
     int H, W;
-    int HB, NB;          // a pixel block: HB rows of NB images at one x (HB NB = 128)
+    int HB, NB;          // a pixel block: HB rows of NB images at one x (HB NB = 64)
     int ytiles;          // pixel blocks per column of an image
     int S;               // stages
     int wrapx;
@@ -772,7 +776,8 @@ struct WgTcArgs {
     unsigned ncol;       // TMEM columns (power of two >= 32, >= cout)
 };
 constexpr int WG_SMAX = 4;
-constexpr int WG_K = 128;                        // pixels per block
+constexpr int WG_BLOCK = 64;                     // pixels per block
+constexpr int WG_K = 2 * WG_BLOCK;               // pixels per stage
 constexpr unsigned WG_ABYTES = 128 * WG_K * 2;   // the x operand: 128 rows
 constexpr unsigned wg_stage_bytes(int cout) { return WG_ABYTES + (unsigned)cout * WG_K * 2; }
 
@@ -797,8 +802,11 @@ __device__ __forceinline__ void tma_load4(unsigned dst, const CUtensorMap *map, 
         : "memory");
 }
 
+// tmX, tmZ: boxes of two columns; tmX1, tmZ1: of one
 __global__ void __launch_bounds__(160) k_wgrad_tc(const WgTcArgs a, const __grid_constant__ CUtensorMap tmX,
-                                                  const __grid_constant__ CUtensorMap tmZ, int *err) {
+                                                  const __grid_constant__ CUtensorMap tmX1,
+                                                  const __grid_constant__ CUtensorMap tmZ,
+                                                  const __grid_constant__ CUtensorMap tmZ1, int *err) {
     extern __shared__ __align__(1024) unsigned char wg_smem[];
     __shared__ __align__(8) unsigned long long full[WG_SMAX], empty[WG_SMAX], done;
     __shared__ unsigned tmem_base;
@@ -816,6 +824,7 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(const WgTcArgs a, const __grid
     const unsigned aatom = WG_K * arow, batom = WG_K * brow;    // bytes of one atom
     const long long kb0 = (long long)blockIdx.x * a.kb_per;
     const int KB = (int)min((long long)a.kb_per, a.kb_total - kb0);  // >= 1
+    const int xstart = (int)(kb0 % a.W);
     if (tid == 0) {
         s_fail = 0;
         s_issued = 0;
@@ -836,31 +845,42 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(const WgTcArgs a, const __grid
     asm volatile("tcgen05.fence::after_thread_sync;");
     const unsigned tmem = uniform(tmem_base);
     if (warp == 0) {
-        // ---- producer: lane j < np loads pair j's x box, the next nb_atoms
+        // ---- producer: lane j < np loads pair j's x boxes, the next nb_atoms
         // lanes the dz boxes (np + nb_atoms <= 12)
-        const unsigned tx = (unsigned)np * aatom + (unsigned)nb_atoms * batom;
+        const unsigned tx = ((unsigned)np * aatom + (unsigned)nb_atoms * batom) / 2;   // bytes of one block
         const bool isx = lane < np, loads = lane < np + nb_atoms;
         const int pr = p0 + lane, tap = pr / cblocks, j = lane - np;
         const int dy = isx ? tap / 3 - 1 : 0, dx = isx ? tap % 3 - 1 : 0;
         const int c0 = isx ? (pr - tap * cblocks) * a.CA : j * a.CB;
-        const unsigned off = isx ? lane * aatom : WG_ABYTES + j * batom;
-        const CUtensorMap *map = isx ? &tmX : &tmZ;
-        int xcol = (int)(kb0 % a.W), yt = (int)(kb0 / a.W % a.ytiles), ng = (int)(kb0 / a.W / a.ytiles);
+        const unsigned off = isx ? lane * aatom : WG_ABYTES + j * batom, second = (isx ? aatom : batom) / 2;
+        const CUtensorMap *map = isx ? &tmX : &tmZ, *map1 = isx ? &tmX1 : &tmZ1;
+        int xcol = xstart, yt = (int)(kb0 / a.W % a.ytiles), ng = (int)(kb0 / a.W / a.ytiles);
         int s = 0, ph = 1;
-        for (int i = 0; i < KB; ++i) {
+        for (int i = 0, stage = 0; i < KB; ++stage) {
+            const bool two = i + 1 < KB && xcol + 1 < a.W;
             if (lane == 0) {
-                if (i >= a.S) ws_wait(&empty[s], ph, &s_fail);
+                if (stage >= a.S) ws_wait(&empty[s], ph, &s_fail);
                 if (!s_fail) {
-                    mbar_expect(&full[s], tx);
-                    s_issued = i + 1;
+                    mbar_expect(&full[s], two ? 2 * tx : tx);
+                    s_issued = stage + 1;
                 }
             }
             if (__shfl_sync(0xffffffffu, lane == 0 && s_fail ? 1 : 0, 0)) break;
-            int xx = xcol + dx;
-            if (a.wrapx) xx = xx < 0 ? xx + a.W : (xx >= a.W ? xx - a.W : xx);
-            if (loads) tma_load4(base + s * STAGE + off, map, c0, xx, yt * a.HB + dy, ng * a.NB, smem_addr(&full[s]));
+            if (loads) {
+                const unsigned dst = base + s * STAGE + off, bar = smem_addr(&full[s]);
+                const int y = yt * a.HB + dy, n = ng * a.NB, x = xcol + dx;
+                if (two && !(a.wrapx && (x < 0 || x + 1 >= a.W))) {
+                    tma_load4(dst, map, c0, y, n, x, bar);
+                } else {
+                    auto column = [&](int v) { return !a.wrapx ? v : (v < 0 ? v + a.W : (v >= a.W ? v - a.W : v)); };
+                    tma_load4(dst, map1, c0, y, n, column(x), bar);
+                    if (two) tma_load4(dst + second, map1, c0, y, n, column(x + 1), bar);
+                }
+            }
             __syncwarp();
-            if (++xcol == a.W) {
+            i += two ? 2 : 1;
+            xcol += two ? 2 : 1;
+            if (xcol == a.W) {
                 xcol = 0;
                 if (++yt == a.ytiles) {
                     yt = 0;
@@ -873,21 +893,30 @@ __global__ void __launch_bounds__(160) k_wgrad_tc(const WgTcArgs a, const __grid
             }
         }
     } else if (warp == 4) {
-        // ---- MMA issuer: M = 128, N = cout, both operands MN-major
+        // ---- MMA issuer: M = 128, N = cout, both operands MN-major; the
+        // stages follow the producer's rule
         const uint32_t idesc = tc_idesc(128, a.cout) | (1u << 15) | (1u << 16);
         const uint64_t ad = tc_desc_mn(0, aatom, 8 * arow, sw_mode_bytes(arow)),
                        bd = tc_desc_mn(0, batom, 8 * brow, sw_mode_bytes(brow));
         const unsigned ahi = (unsigned)(ad >> 32), bhi = (unsigned)(bd >> 32);
         const unsigned a16 = (unsigned)ad + (base >> 4), b16 = (unsigned)bd + ((base + WG_ABYTES) >> 4);
-        int s = 0, ph = 0;
-        for (int i = 0; i < KB; ++i) {
+        int s = 0, ph = 0, xcol = xstart;
+        for (int i = 0; i < KB;) {
+            const bool two = i + 1 < KB && xcol + 1 < a.W;
             ws_wait(&full[s], ph, &s_fail);
             asm volatile("tcgen05.fence::after_thread_sync;");
             const unsigned as = a16 + s * (STAGE >> 4), bs = b16 + s * (STAGE >> 4);
 #pragma unroll
-            for (int ks = 0; ks < WG_K / 16; ++ks)
+            for (int ks = 0; ks < WG_BLOCK / 16; ++ks)
                 mma_elect(tmem, as + ks * arow, bs + ks * brow, ahi, bhi, idesc, ks > 0 ? 1u : (unsigned)i);
+            if (two)
+#pragma unroll
+                for (int ks = WG_BLOCK / 16; ks < WG_K / 16; ++ks)
+                    mma_elect(tmem, as + ks * arow, bs + ks * brow, ahi, bhi, idesc, 1u);
             commit_elect(smem_addr(&empty[s]));
+            i += two ? 2 : 1;
+            xcol += two ? 2 : 1;
+            if (xcol == a.W) xcol = 0;
             if (++s == a.S) {
                 s = 0;
                 ph ^= 1;
@@ -1901,20 +1930,21 @@ lbm_status bias_grad(lbm_unet *u, const bf16 *dz, int dzc, int C, long long P, f
     return LBM_OK;
 }
 
-// The tcgen05 weight gradient when the shape suits its pixel blocks (H a
-// divisor of 128, or above 128) and every global address and stride is a
-// multiple of 16 bytes.  Returns false (nothing launched) otherwise, and when
-// a tensor map cannot be made.  The pixel blocks are split into about two CTAs
-// per SM, also where only one fits at a time, each taking at least 4 blocks
-// (its 128 x N atomics stay small against its MMA work).  The split sets the
-// length of the FP32 sums in TMEM, whose additions truncate: with one CTA per
-// SM for the wide layers the gradient moved by 8e-7 relative, twice this split
-// costs 5 % of a training step (128 x 256, batch 8: 1.37 and 1.44 ms).
+// The tcgen05 weight gradient when the shape suits its pixel blocks (64
+// pixels of one column: H <= 64 dividing 64 with n a multiple of 64 / H, or H
+// a multiple of 64) and every global address and stride is a multiple of 16
+// bytes.  Returns false (nothing launched) otherwise, and when a tensor map
+// cannot be made.  The pixel blocks are split into about two CTAs per SM, also
+// where only one fits at a time, each taking at least 8 blocks (its 128 x N
+// atomics stay small against its MMA work).  The split sets the length of the
+// FP32 sums in TMEM, whose additions truncate: with one CTA per SM for the
+// wide layers the gradient moved by 8e-7 relative, twice this split costs 5 %
+// of a training step (128 x 256, batch 8: 1.37 and 1.44 ms).
 bool launch_wgrad_tc(lbm_unet *u, const Layer &l, const bf16 *dz, int dzc, const bf16 *x, int xc, int xo, int n,
                      int H, int W, lbm_status *st) {
-    const int HB = H <= WG_K ? H : WG_K;
-    const int NB = WG_K / HB;
-    if (WG_K % HB != 0) return false;
+    const int HB = H <= WG_BLOCK ? H : WG_BLOCK;
+    const int NB = WG_BLOCK / HB;
+    if (H <= WG_BLOCK ? (WG_BLOCK % H != 0 || n % NB != 0) : (H % WG_BLOCK != 0)) return false;
     const int cin = l.cinp, cout = l.coutp;
     // atom widths are swizzle widths: 16, 32 or 64 channels
     if ((cin < 64 ? (cin != 16 && cin != 32) : cin % 64 != 0) || cout > 256 || (cout < 64 ? cout != 32 : cout % 64 != 0))
@@ -1928,22 +1958,20 @@ bool launch_wgrad_tc(lbm_unet *u, const Layer &l, const bf16 *dz, int dzc, const
     auto swz = [](int ch) {
         return ch == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : (ch == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
     };
-    alignas(64) CUtensorMap tx, tz;
-    const cuuint32_t es[4] = {1u, 1u, 1u, 1u};
-    const cuuint64_t gdX[4] = {(cuuint64_t)cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)n};
-    const cuuint64_t rx = (cuuint64_t)xc * 2;
-    const cuuint64_t gsX[3] = {rx, rx * W, rx * W * H};
-    const cuuint32_t boxX[4] = {(cuuint32_t)CA, 1u, (cuuint32_t)HB, (cuuint32_t)NB};
-    if (enc(&tx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)(x + xo), gdX, gsX, boxX, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, swz(CA), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return false;
-    const cuuint64_t gdZ[4] = {(cuuint64_t)cout, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)n};
-    const cuuint64_t rz = (cuuint64_t)dzc * 2;
-    const cuuint64_t gsZ[3] = {rz, rz * W, rz * W * H};
-    const cuuint32_t boxZ[4] = {(cuuint32_t)CB, 1u, (cuuint32_t)HB, (cuuint32_t)NB};
-    if (enc(&tz, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)dz, gdZ, gsZ, boxZ, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            swz(CB), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    // NHWC as (channel, y, image, x), so that a box of two columns is laid out
+    // column after column
+    auto columns = [&](CUtensorMap *m, const bf16 *p, int ch, int stride, int atom, int cols) {
+        const cuuint32_t es[4] = {1u, 1u, 1u, 1u};
+        const cuuint64_t pix = (cuuint64_t)stride * 2;
+        const cuuint64_t gd[4] = {(cuuint64_t)ch, (cuuint64_t)H, (cuuint64_t)n, (cuuint64_t)W};
+        const cuuint64_t gs[3] = {pix * W, pix * W * H, pix};
+        const cuuint32_t box[4] = {(cuuint32_t)atom, (cuuint32_t)HB, (cuuint32_t)NB, (cuuint32_t)cols};
+        return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)p, gd, gs, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   swz(atom), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    alignas(64) CUtensorMap tx, tx1, tz, tz1;
+    if (!columns(&tx, x + xo, cin, xc, CA, 2) || !columns(&tx1, x + xo, cin, xc, CA, 1) ||
+        !columns(&tz, dz, cout, dzc, CB, 2) || !columns(&tz1, dz, cout, dzc, CB, 1))
         return false;
     WgTcArgs a{};
     a.dw = u->g + l.woff;
@@ -1957,15 +1985,15 @@ bool launch_wgrad_tc(lbm_unet *u, const Layer &l, const bf16 *dz, int dzc, const
     a.CA = CA;
     a.CB = CB;
     a.pairs = 9 * cin / CA;
-    a.ytiles = (H + HB - 1) / HB;
-    a.kb_total = (long long)((n + NB - 1) / NB) * a.ytiles * W;
+    a.ytiles = H / HB;
+    a.kb_total = (long long)n * H * W / WG_BLOCK;
     a.ncol = cout <= 32 ? 32u : (cout <= 64 ? 64u : (cout <= 128 ? 128u : 256u));
     const int mtiles = (a.pairs + 128 / CA - 1) / (128 / CA);
     const size_t stage = wg_stage_bytes(cout), half = 233472 / 2 - 2048;
     const int ctas = 2 * stage <= half ? 2 : 1;   // per SM
     a.S = (int)std::min<size_t>(WG_SMAX, (ctas == 2 ? half : (size_t)229376) / stage);
     long long splits = (2LL * u->sms + mtiles - 1) / mtiles;
-    const long long cap = a.kb_total / 4 > 0 ? a.kb_total / 4 : 1;
+    const long long cap = a.kb_total / 8 > 0 ? a.kb_total / 8 : 1;
     if (splits > cap) splits = cap;
     a.kb_per = (int)((a.kb_total + splits - 1) / splits);
     splits = (a.kb_total + a.kb_per - 1) / a.kb_per;  // every CTA gets at least one block
@@ -1980,7 +2008,7 @@ bool launch_wgrad_tc(lbm_unet *u, const Layer &l, const bf16 *dz, int dzc, const
         attr = true;
     }
     const size_t need = a.S * stage + 1024;
-    k_wgrad_tc<<<dim3((unsigned)splits, (unsigned)mtiles), 160, need, u->stream>>>(a, tx, tz, u->tc_err);
+    k_wgrad_tc<<<dim3((unsigned)splits, (unsigned)mtiles), 160, need, u->stream>>>(a, tx, tx1, tz, tz1, u->tc_err);
     cudaError_t e = cudaGetLastError();
     *st = e == cudaSuccess ? LBM_OK : ufail(u, LBM_ERR_CUDA, std::string("k_wgrad_tc: ") + cudaGetErrorString(e));
     return true;
