@@ -1330,7 +1330,7 @@ __global__ void __launch_bounds__(384) k_conv_col(const ConvArgs a, const __grid
 // shared memory and each channel's sum goes out in one atomic.  Channels
 // C .. 8 G - 1 are read (the buffer has them: its stride is a multiple of 8)
 // but never written.
-constexpr int kBiasLoads = 8;   // loads per thread and block, all in flight at once
+constexpr int kBiasLoads = 16;  // loads per thread and block: the terms of one FP32 sum
 __global__ void __launch_bounds__(256) k_bias_grad(const bf16 *dz, int dzc, int C, long long P, int chunk, float *db) {
     __shared__ float sh[256 * 8];
     const int G = (C + 7) >> 3, R = 256 / G;

@@ -106,3 +106,16 @@ def test_weight_gradient_sums(H, W, n, image, x0):
         if g[wo + 4 * ci] != want:
             bad[name] = (g[wo + 4 * ci], want)
     assert not bad, bad
+
+
+def test_bias_gradient_sums():
+    """The head's bias: a thread adds 16 pixels 256 apart, in FP32."""
+    import paper_2212_07494_gb300 as P
+    net, sl = _copy_net(P, 128, 256, 1)
+    bo = sl[-1][5]
+    for first, thread in ((0, 0), (4096, 77), (28672, 255)):
+        m = np.ones(128 * 256)
+        m[first + thread] = BIG
+        m[first + thread + 15 * 256] = -BIG
+        assert _grad(net, m.reshape(1, 128, 256))[bo] == 128 * 256 - 16, (first, thread)
+    net.close()
