@@ -1541,14 +1541,17 @@ struct PackArgs {
     int step;
     float lr, b1, b2, eps, c1, c2;
 };
+// The fused multiply-adds are written out: left to the compiler, which of a
+// moment's two products is rounded before the sum depends on the code around
+// it, and a weight's last bit, sent through the next steps, with it.
 __device__ __forceinline__ float adam_step(const PackArgs &a, long long i) {
     if (!a.step) return a.p[i];
     const float gi = a.g[i];
-    const float mi = a.b1 * a.m[i] + (1.f - a.b1) * gi;
-    const float vi = a.b2 * a.v[i] + (1.f - a.b2) * gi * gi;
+    const float mi = __fmaf_rn(1.f - a.b1, gi, __fmul_rn(a.b1, a.m[i]));
+    const float vi = __fmaf_rn(__fmul_rn(1.f - a.b2, gi), gi, __fmul_rn(a.b2, a.v[i]));
     a.m[i] = mi;
     a.v[i] = vi;
-    const float pn = a.p[i] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
+    const float pn = __fsub_rn(a.p[i], a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps));
     a.p[i] = pn;
     return pn;
 }

@@ -119,3 +119,34 @@ def test_bias_gradient_sums():
         m[first + thread + 15 * 256] = -BIG
         assert _grad(net, m.reshape(1, 128, 256))[bo] == 128 * 256 - 16, (first, thread)
     net.close()
+
+
+def test_adam_rounding():
+    """Four Adam steps from the library's own gradients and parameters: both moments add a rounded product of the old
+    moment to an exact one of the gradient (one fused multiply-add), every other operation is rounded on its own.
+    Emulated in extended precision with a rounding to FP32 after each operation: equal bit for bit (products of two
+    FP32 values and their sum with a third round the same from 64 bits of mantissa but for ties of one in 2^40)."""
+    import torch
+    import paper_2212_07494_gb300 as P
+    f, L = np.float32, np.longdouble
+    if np.finfo(L).nmant < 63:
+        pytest.skip("no extended precision")
+    H, W, n = 32, 64, 2
+    rng = np.random.default_rng(1)
+    net = P.UNet(H, W, n, cin=3)
+    net.set_params(0.05 * rng.normal(size=net.n))
+    x, t = (torch.tensor(rng.normal(size=(n, H, W, 3)), dtype=torch.float32, device="cuda") for _ in range(2))
+    w = torch.ones((n, H, W), device="cuda")
+    b1, b2, lr, eps = f(0.9), f(0.999), f(1e-3), f(1e-8)
+    o1, o2 = f(1) - b1, f(1) - b2
+    m, v = np.zeros(net.n, f), np.zeros(net.n, f)
+    for k in range(1, 5):
+        p = net.params().copy()
+        g = np.asarray(net.grad(x.data_ptr(), t.data_ptr(), w.data_ptr(), n, 1 / (3.0 * n * H * W))[1], f)
+        net.adam(float(lr))
+        m = (L(o1) * g + L(1) * (b1 * m)).astype(f)
+        v = ((o2 * g).astype(L) * g + L(1) * (b2 * v)).astype(f)
+        c1, c2 = f(1) - f(float(b1) ** k), f(1) - f(float(b2) ** k)
+        want = p - (lr * (m / c1)) / (np.sqrt(v / c2) + eps)
+        assert np.array_equal(net.params(), want), (k, np.mean(net.params() != want))
+    net.close()
