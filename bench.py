@@ -415,9 +415,12 @@ def run_gpu(args, ws, rank, local):
     traffic = (traffic_per_launch(N, coll)
                if st == "F32" and not args.tau_bulk and spec["lattice"] == "D2Q9" and K == 1 else None)
     clocks = sampler.summary()
-    # step kernels (runs of n steps: K per launch, what is left over in smaller ones), and the moments and finalize
-    # kernels per check
-    launches = sum(n // K + (n % K) // 2 + (n % K) % 2 if K > 1 else n for _, _, n in chunk_ev) + 2 * k
+    # step kernels (runs of n steps: K per launch, what is left over in smaller ones, one more where the launches would
+    # differ from the steps by an odd number), and the moments and finalize kernels per check
+    launches = 2 * k
+    for _, _, n in chunk_ev:
+        m = n // K + (n % K) // 2 + (n % K) % 2 if K > 1 else n
+        launches += m + (n - m) % 2
 
     e2e = None
     if not args.no_e2e:

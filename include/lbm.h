@@ -127,7 +127,11 @@ typedef struct {
 lbm_status lbm_create(const lbm_desc *desc, lbm_handle **out);
 
 /* Advance nsteps time steps (fused pull-stream, collide, store; Sec. II.B-C).
- * Asynchronous; long runs replay a captured CUDA graph. */
+ * Asynchronous; long runs replay a captured CUDA graph.  The state moves to
+ * the handle's other buffer once per step, however many steps a launch takes:
+ * a caller's own capture of an even number of steps, of lbm_moments_device or
+ * of lbm_check_device (each called once before, outside the capture) can be
+ * replayed after any even number of direct steps. */
 lbm_status lbm_step(lbm_handle *h, int64_t nsteps);
 
 /* Macroscopic fields at the current step (Eq. half_F): rho (nx*ny*nz), u

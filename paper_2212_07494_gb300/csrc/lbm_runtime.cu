@@ -324,14 +324,25 @@ cudaError_t launch_tile(lbm_handle *h, int K, const float *g32, long long g_step
 }
 
 // n <= 64 steps whose forces lie g_step values apart from g / g32 on (0: one
-// force for all)
+// force for all).  The launches are as many as the steps or fewer by an even
+// number (one launch of several steps is halved where need be): the state
+// then lies in the buffer that single steps would leave it in, which a
+// caller's captured steps, moments and checks rely on.
 lbm_status launch_run(lbm_handle *h, int n, double *g, float *g32, long long g_step) {
     KParams &p = h->kp;
     double *const g0 = const_cast<double *>(p.g);
     float *const g320 = const_cast<float *>(p.g32);
     cudaError_t e = cudaSuccess;
-    for (int s = 0; s < n && e == cudaSuccess;) {
-        const int k = fused_steps(h, n - s);
+    int launches = 0;
+    for (int s = 0; s < n; ++launches) s += fused_steps(h, n - s);
+    bool halve = ((n - launches) & 1) != 0;
+    for (int s = 0, half = 0; s < n && e == cudaSuccess;) {
+        int k = half ? half : fused_steps(h, n - s);
+        half = 0;
+        if (halve && k > 1) {
+            halve = false;
+            half = k /= 2;
+        }
         const void *fin = h->buf[h->cur];
         void *fout = h->buf[1 - h->cur];
         if (k > 1) {
@@ -432,7 +443,7 @@ lbm_status ensure_graph(lbm_handle *h) {
     LBM_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
     lbm_status st = launch_steps(h, steps);
     cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-    h->cur = saved;  // capture does not execute, and its launches are even in number
+    h->cur = saved;  // capture does not execute; the launches of an even number of steps are even in number
     if (st != LBM_OK) {
         if (g) cudaGraphDestroy(g);
         return st;
@@ -831,8 +842,7 @@ lbm_status lbm_step(lbm_handle *h, int64_t nsteps) {
             left -= h->graph_steps;
         }
     }
-    // into a caller's own capture, one step per launch: a replay of an even
-    // number of steps then ends in the buffer it began in
+    // into a caller's own capture, one step per launch
     h->hold_fuse = cs != cudaStreamCaptureStatusNone;
     lbm_status st = launch_steps(h, left);
     h->hold_fuse = false;
