@@ -167,11 +167,6 @@ struct KParams {
     const double *g;               // uniform [3] | rows [ny][D] | field [D][plane]
     const float *g32;              // the same force in FP32 (for FP32 arithmetic)
     const unsigned char *solid;    // [plane] or null
-    // obstacle links [plane], made from the mask once (with it or null): bit
-    // i, population i of the node is pulled from a solid node, i.e. bounces
-    // back; bit 0, the node itself is solid.  One load per node instead of
-    // one mask byte per population.
-    const unsigned *links;
     double om[5];                  // 1 / tau_n
     float om32[5];
     double omb;                    // 1 / tau of the trace (bulk) part of order 2; om[2] unless split
@@ -189,6 +184,11 @@ struct KParams {
     // (the node itself, or its neighbour along x, wrapped on a periodic x):
     long long doff[27];            // i*plane - (cy*nxp + cz*nxp*ny): pull source
     long long poff[27];            // i*plane: the node's own entry (relative to the node)
+    // obstacle links [plane], made from the mask once (with it or null): bit
+    // i, population i of the node is pulled from a solid node, i.e. bounces
+    // back; bit 0, the node itself is solid.  One load per node instead of
+    // one mask byte per population.
+    const unsigned *links;
 };
 
 // fill the per-population offsets of KParams for lattice L (host side)
@@ -268,8 +268,18 @@ template <int L, typename R> __host__ __device__ __forceinline__ void reconstruc
     }
 }
 
-// 1 / rho; the pair type has an overload of its own (lbm_f32x2.cuh)
+// 1 / rho; the pair type has an overload of its own (lbm_f32x2.cuh), which RCP
+// selects: the same bits, but other code around it.  Kernels that keep many
+// nodes' values in registers spill more with it, masked k_step and the kernels
+// for several steps run faster (us per step, division and reciprocal:
+// k_step_vec D3Q27 FP32 256^3 575 and 581, D3Q27 FP16 256^2 x 200 271 and 310,
+// D3Q19 BF16 208 and 215, D2Q9 SMRT FP16 4096^2 103 and 109; masked k_step
+// D3Q19 BF16 320 x 128 x 96 150 and 142).
 template <typename R> __host__ __device__ __forceinline__ R one_over(R rho) { return R(1) / rho; }
+template <bool RCP, typename R> __host__ __device__ __forceinline__ R inverse(R rho) {
+    if constexpr (RCP) return one_over(rho);
+    else return R(1) / rho;
+}
 
 // ------------------------------------------------------------------ collisions
 // Second-order central moments scaled by (1 - a) in their traceless (shear)
@@ -293,7 +303,7 @@ template <int D, typename R> __host__ __device__ __forceinline__ void relax_orde
 // G holds the deviations delta on the velocity grid (zeros off-lattice) and is
 // overwritten with the post-collision deviations.  g: acceleration (lattice
 // units).  Returns nothing; rho/u are recomputed by the moments kernel.
-template <int L, typename R>
+template <int L, bool RCP = true, typename R>
 __host__ __device__ __forceinline__ void collide_smrt(R *G, R gx, R gy, R gz, R om2, R om3, R om4, R omb) {
     constexpr int D = Lat<L>::D;
     constexpr int N = Grid<D>::N;
@@ -301,7 +311,7 @@ __host__ __device__ __forceinline__ void collide_smrt(R *G, R gx, R gy, R gz, R 
     project<D>(G);
     const R drho = G[0];                 // rho - 1 (moments of w vanish beyond order 0)
     const R rho = R(1) + drho;
-    const R inv = one_over(rho);
+    const R inv = inverse<RCP>(rho);
     const R ux = G[EX] * inv + R(0.5) * gx;   // Eq. (half_F)
     const R uy = G[EY] * inv + R(0.5) * gy;
     const R uz = D == 3 ? G[EZ] * inv + R(0.5) * gz : R(0);
@@ -451,7 +461,7 @@ __host__ __device__ __forceinline__ void shift_pass(R *a, R v) {
 // SMRT with tau_3 = tau_4 = 1 (om3 = om4 = 1): the same collision as
 // collide_smrt, whose orders-3/4 factors (1 - om) are then exactly zero,
 // with the passes restricted to what is non-zero or read.
-template <int L, typename R>
+template <int L, bool RCP = true, typename R>
 __host__ __device__ __forceinline__ void collide_smrt_trim(R *G, R gx, R gy, R gz, R om2) {
     constexpr int D = Lat<L>::D;
     constexpr int N = Grid<D>::N;
@@ -468,7 +478,7 @@ __host__ __device__ __forceinline__ void collide_smrt_trim(R *G, R gx, R gy, R g
     if constexpr (D == 3) proj_pass<D, 2, P3>(G);
     const R drho = G[0];
     const R rho = R(1) + drho;
-    const R inv = one_over(rho);
+    const R inv = inverse<RCP>(rho);
     const R ux = G[EX] * inv + R(0.5) * gx;   // Eq. (half_F)
     const R uy = G[EY] * inv + R(0.5) * gy;
     const R uz = D == 3 ? G[EZ] * inv + R(0.5) * gz : R(0);
@@ -517,7 +527,7 @@ __host__ __device__ __forceinline__ void collide_smrt_trim(R *G, R gx, R gy, R g
 // Eq. (newf) inverts to d^(n) = (1 - om_n/2)(dbar_1^(n) + d_F^(n)/2).  Hence
 // d_F^(2) = 0, d_F^(3) = 3 g d^(2) and d_F^(4) = 4 g d^(3), each order needing
 // the one below it.  Relaxation as in collide_smrt with these d_F added.
-template <int L, typename R>
+template <int L, bool RCP = true, typename R>
 __host__ __device__ __forceinline__ void collide_smrt_fneq(R *G, R gx, R gy, R gz, R om2, R om3, R om4, R omb) {
     constexpr int D = Lat<L>::D;
     constexpr int N = Grid<D>::N;
@@ -525,7 +535,7 @@ __host__ __device__ __forceinline__ void collide_smrt_fneq(R *G, R gx, R gy, R g
     project<D>(G);
     const R drho = G[0];
     const R rho = R(1) + drho;
-    const R inv = one_over(rho);
+    const R inv = inverse<RCP>(rho);
     const R ux = G[EX] * inv + R(0.5) * gx;   // Eq. (half_F)
     const R uy = G[EY] * inv + R(0.5) * gy;
     const R uz = D == 3 ? G[EZ] * inv + R(0.5) * gz : R(0);
@@ -584,7 +594,7 @@ __host__ __device__ __forceinline__ void collide_smrt_fneq(R *G, R gx, R gy, R g
 // recursion is the statement that the fourth-order central moment of the
 // non-equilibrium part vanishes, so it is applied as a round trip through
 // the co-moving frame with the orders >= 4 dropped.
-template <int L, typename R>
+template <int L, bool RCP = true, typename R>
 __host__ __device__ __forceinline__ void collide_mrt_raw(R *G, R gx, R gy, R gz, R om2, R om3, R om4) {
     constexpr int D = Lat<L>::D;
     constexpr int N = Grid<D>::N;
@@ -592,7 +602,7 @@ __host__ __device__ __forceinline__ void collide_mrt_raw(R *G, R gx, R gy, R gz,
     project<D>(G);
     const R drho = G[0];
     const R rho = R(1) + drho;
-    const R inv = one_over(rho);
+    const R inv = inverse<RCP>(rho);
     const R ux = G[EX] * inv + R(0.5) * gx;   // Eq. (half_F)
     const R uy = G[EY] * inv + R(0.5) * gy;
     const R uz = D == 3 ? G[EZ] * inv + R(0.5) * gz : R(0);
@@ -640,7 +650,7 @@ __host__ __device__ __forceinline__ void collide_mrt_raw(R *G, R gx, R gy, R gz,
 }
 
 // BGK with the second-order equilibrium and Guo-form force, Eq. (explict_eq)
-template <int L, typename R>
+template <int L, bool RCP = true, typename R>
 __host__ __device__ __forceinline__ void collide_bgk(R *G, R gx, R gy, R gz, R om) {
     constexpr int Q = Lat<L>::Q;
     constexpr int D = Lat<L>::D;
@@ -654,7 +664,7 @@ __host__ __device__ __forceinline__ void collide_bgk(R *G, R gx, R gy, R gz, R o
         if (D == 3 && Lat<L>::cz(i)) jz += Lat<L>::cz(i) > 0 ? v : -v;
     }
     const R rho = R(1) + drho;
-    const R inv = one_over(rho);
+    const R inv = inverse<RCP>(rho);
     const R ux = jx * inv + R(0.5) * gx, uy = jy * inv + R(0.5) * gy;
     const R uz = D == 3 ? jz * inv + R(0.5) * gz : R(0);
     const R uu15 = R(1.5) * (ux * ux + uy * uy + uz * uz);

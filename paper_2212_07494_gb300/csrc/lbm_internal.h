@@ -15,17 +15,17 @@
 namespace lbm {
 
 // the collision selected by COLL on one node's grid G (or two nodes' with F2)
-template <int L, int COLL, typename R>
+template <int L, int COLL, bool RCP = true, typename R>
 __device__ __forceinline__ void collide_any(R *G, R gx, R gy, R gz, R om2, R om3, R om4, R omb) {
     // FP64: the forms with fewer FP64 instructions (lbm_collide64.cuh)
     if constexpr (std::is_same<R, double>::value && COLL == BGK) collide_bgk64<L>(G, gx, gy, gz, om2);
     else if constexpr (std::is_same<R, double>::value && COLL == SMRT_TRIM && L == D2Q9)
         collide_smrt_trim64(G, gx, gy, om2);
-    else if constexpr (COLL == SMRT) collide_smrt<L>(G, gx, gy, gz, om2, om3, om4, omb);
-    else if constexpr (COLL == SMRT_TRIM) collide_smrt_trim<L>(G, gx, gy, gz, om2);
-    else if constexpr (COLL == SMRT_FNEQ) collide_smrt_fneq<L>(G, gx, gy, gz, om2, om3, om4, omb);
-    else if constexpr (COLL == MRT_RAW) collide_mrt_raw<L>(G, gx, gy, gz, om2, om3, om4);
-    else collide_bgk<L>(G, gx, gy, gz, om2);
+    else if constexpr (COLL == SMRT) collide_smrt<L, RCP>(G, gx, gy, gz, om2, om3, om4, omb);
+    else if constexpr (COLL == SMRT_TRIM) collide_smrt_trim<L, RCP>(G, gx, gy, gz, om2);
+    else if constexpr (COLL == SMRT_FNEQ) collide_smrt_fneq<L, RCP>(G, gx, gy, gz, om2, om3, om4, omb);
+    else if constexpr (COLL == MRT_RAW) collide_mrt_raw<L, RCP>(G, gx, gy, gz, om2, om3, om4);
+    else collide_bgk<L, RCP>(G, gx, gy, gz, om2);
 }
 
 // One node's collision.  In FP32 the node runs through the pair type with
@@ -33,18 +33,18 @@ __device__ __forceinline__ void collide_any(R *G, R gx, R gy, R gz, R om2, R om3
 // template instantiation and the same instructions as two paired nodes, so
 // a node's result does not depend on whether the launch shape collides it
 // alone or paired.  FP64 as written.
-template <int L, int COLL, typename R>
+template <int L, int COLL, bool RCP = true, typename R>
 __device__ __forceinline__ void collide_one(R *G, R gx, R gy, R gz, R om2, R om3, R om4, R omb) {
     if constexpr (sizeof(R) == 4) {
         constexpr int NG = Grid<Lat<L>::D>::N;
         F2 H[NG];
 #pragma unroll
         for (int g = 0; g < NG; ++g) H[g] = F2(G[g]);
-        collide_any<L, COLL>(H, F2(gx), F2(gy), F2(gz), F2(om2), F2(om3), F2(om4), F2(omb));
+        collide_any<L, COLL, RCP>(H, F2(gx), F2(gy), F2(gz), F2(om2), F2(om3), F2(om4), F2(omb));
 #pragma unroll
         for (int g = 0; g < NG; ++g) G[g] = H[g].lo();
     } else {
-        collide_any<L, COLL>(G, gx, gy, gz, om2, om3, om4, omb);
+        collide_any<L, COLL, RCP>(G, gx, gy, gz, om2, om3, om4, omb);
     }
 }
 

@@ -31,7 +31,7 @@ __device__ __noinline__ void step_node_alone(const KParams &p, const typename St
     const long long own = node_index(p, x, y, z);
     R gx, gy, gz;
     load_force<L>(p, y, own, gx, gy, gz);
-    collide_one<L, COLL>(G, gx, gy, gz, omega<R>(p, 2), omega<R>(p, 3), omega<R>(p, 4), omega_bulk<R>(p));
+    collide_one<L, COLL, MASK>(G, gx, gy, gz, omega<R>(p, 2), omega<R>(p, 3), omega<R>(p, 4), omega_bulk<R>(p));
     typename Store<ST>::T *dst = fout + own;
 #pragma unroll
     for (int i = 0; i < Lat<L>::Q; ++i) Store<ST>::st(dst + p.poff[i], G[gpos<L>(i)]);
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(256, step_min_blocks<ST>()) k_step(const __gri
                 gy2 = F2::pair(ay, by);
                 gz2 = F2::pair(az, bz);
             }
-            collide_any<L, COLL>(G2, gx2, gy2, gz2, F2(om2), F2(om3), F2(om4), F2(omb));
+            collide_any<L, COLL, MASK>(G2, gx2, gy2, gz2, F2(om2), F2(om3), F2(om4), F2(omb));
             typename Store<ST>::T *d0 = fout + own0, *d1 = fout + own1;
 #pragma unroll
             for (int i = 0; i < Lat<L>::Q; ++i) {
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(256, step_min_blocks<ST>()) k_step(const __gri
             const int x = x0 + k * blockDim.x;
             const long long own = node_index(p, x, y, z);
             if (per_node_force) load_force<L>(p, y, own, gx, gy, gz);
-            collide_one<L, COLL>(G[k], gx, gy, gz, om2, om3, om4, omb);
+            collide_one<L, COLL, MASK>(G[k], gx, gy, gz, om2, om3, om4, omb);
             typename Store<ST>::T *dst = fout + own;
 #pragma unroll
             for (int i = 0; i < Lat<L>::Q; ++i) Store<ST>::st(dst + p.poff[i], G[k][gpos<L>(i)]);

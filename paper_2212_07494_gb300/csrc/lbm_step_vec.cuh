@@ -214,7 +214,7 @@ __device__ __forceinline__ void step_vec_nodes(const KParams &p, const typename 
                 gy2 = F2::pair(ay, by);
                 gz2 = F2::pair(az, bz);
             }
-            collide_any<L, COLL>(G2, gx2, gy2, gz2, F2(om2), F2(om3), F2(om4), F2(omb));
+            collide_any<L, COLL, false>(G2, gx2, gy2, gz2, F2(om2), F2(om3), F2(om4), F2(omb));
             typename Store<ST>::T *dst = fout + own;
 #pragma unroll
             for (int i = 0; i < Q; ++i) {
@@ -231,7 +231,7 @@ __device__ __forceinline__ void step_vec_nodes(const KParams &p, const typename 
             gather<L, ST, false>(p, fin, x, y, z, G);
             const long long own = node_index(p, x, y, z);
             if (per_node_force) load_force<L>(p, y, own, gx, gy, gz);
-            collide_one<L, COLL>(G, gx, gy, gz, om2, om3, om4, omb);
+            collide_one<L, COLL, false>(G, gx, gy, gz, om2, om3, om4, omb);
             typename Store<ST>::T *dst = fout + own;
 #pragma unroll
             for (int i = 0; i < Q; ++i) Store<ST>::st(dst + p.poff[i], G[gpos<L>(i)]);
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(256, vec_min_blocks<L, ST>()) k_step_vec(const
                         gy2 = F2::pair(ay, by);
                         gz2 = F2::pair(az, bz);
                     }
-                    collide_any<L, COLL>(G2, gx2, gy2, gz2, F2(om2), F2(om3), F2(om4), F2(omb));
+                    collide_any<L, COLL, false>(G2, gx2, gy2, gz2, F2(om2), F2(om3), F2(om4), F2(omb));
 #pragma unroll
                     for (int i = 0; i < Q; ++i) {
                         VT::put(o[i], k, G2[gpos<L>(i)].lo(), held[i]);
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(256, vec_min_blocks<L, ST>()) k_step_vec(const
                         G[gpos<L>(i)] = (e < 0 || e >= V) ? dec<ST>(edge[i]) : VT::delem(w[i], e);
                     }
                     if (per_node_force) load_force<L>(p, y, (long long)own + k, gx, gy, gz);
-                    collide_one<L, COLL>(G, gx, gy, gz, om2, om3, om4, omb);
+                    collide_one<L, COLL, false>(G, gx, gy, gz, om2, om3, om4, omb);
 #pragma unroll
                     for (int i = 0; i < Q; ++i) VT::put(o[i], k, G[gpos<L>(i)], held[i]);
                 }
