@@ -233,7 +233,8 @@ lbm_status lbm_set_launch(lbm_handle *h, int block_x, int nodes_per_thread);
 /* The current launch shape (outputs nullable). */
 lbm_status lbm_get_launch(const lbm_handle *h, int *block_x, int *nodes_per_thread, int *layout);
 /* Time steps that one kernel launch of a long lbm_step advances: 2 or 4 on a
- * new D2Q9 handle in FP32, FP16 or BF16 storage (the steps between kept in
+ * new D2Q9 handle in FP32 storage, and in FP16 or BF16 storage where that is
+ * measured faster (the steps between kept in
  * shared memory; bit for bit the result of single steps, to which lbm_step
  * falls back for what is left over), else 1.  lbm_set_launch and
  * lbm_set_launch_layout set 1; lbm_autotune keeps what it measures faster. */

@@ -288,6 +288,34 @@ bool tile_ok(const lbm_handle *h) {
            (long long)h->Q * h->kp.plane * (long long)storage_bytes(h->storage) < (1LL << 32);
 }
 
+// Whether two steps per launch are faster than single ones on a domain of
+// more than 1.5e5 nodes.  They are in FP32, with an obstacle mask, with walls
+// or a ragged width (a single step then takes a second launch for those
+// nodes) and with a force per node (us per step, single and two, the closest
+// of each: 1024^2 FP32 10.0 / 7.7, 4096^2 FP16 with cylinders 282 / 152, with
+// walls 87.9 / 76.3 (3072^2), 4095 x 4096 150 / 123, force per node 135 / 126).
+// Without any of these the vector kernel's single step in 2-byte storage is
+// bound by its collisions while both buffers (36 bytes per node) lie in the
+// 129 MB L2, and two steps add the margins' collisions: they win up to 1e6
+// nodes (768^2 5.2 / 5.0, 1000^2 7.4 / 7.1 and, MRT_RAW, 9.8 / 9.1; BGK, the
+// longest single step, to 2e6: 1280^2 15.4 / 14.4) and lose above (1280^2
+// 10.1 / 10.4, 1536^2 13.6 / 14.5 - 18.1 / 18.9, 512 x 4096 12.2 / 13.8 and,
+// BGK, 18.7 / 19.1).  Past L2 a single step waits for memory: two steps win for
+// the trimmed SMRT (1840^2 21.8 / 20.4, 4096^2 95.1 / 91.4, 8192^2 375 / 370),
+// for the longer collisions just past it (1840^2 28.1 / 26.3, 2048^2 32.8 /
+// 32.1) but not far beyond (2304^2 39.6 / 39.7, 4096^2 102 / 106 - 113 / 122).
+bool two_steps_pay(const lbm_handle *h) {
+    const KParams &p = h->kp;
+    const long long n = (long long)h->nx * h->ny;
+    if (h->storage == LBM_F32 || h->mask || h->force_kind == LBM_G_FIELD || !p.per[0] || !p.per[1] ||
+        h->nx % vec_width_hi(h->lattice, h->storage) != 0)
+        return true;
+    if (n <= (h->collision == LBM_BGK ? 2000000 : 1000000)) return true;
+    if (n < 3300000) return false;
+    const bool trim = h->collision == LBM_SMRT && p.om[3] == 1.0 && p.om[4] == 1.0 && p.omb == p.om[2];
+    return trim || n < 4500000;
+}
+
 // Steps of one launch when `left` are wanted.  Small domains take four per
 // launch: a launch's latency (about 2.3 us for two steps) bounds them, and
 // the margins' extra collisions are hidden.  From about 1.5e5 nodes on the
@@ -295,8 +323,9 @@ bool tile_ok(const lbm_handle *h) {
 // against two: 400 x 300 1.82 / 1.95, 512^2 2.95 / 2.82, 1024^2 9.3 / 7.4).
 int fused_steps(const lbm_handle *h, int64_t left) {
     if (!h->fuse || h->hold_fuse || !tile_ok(h) || (h->gs_dev && !h->gring_dev)) return 1;
-    if (left >= 4 && (long long)h->nx * h->ny <= 150000) return 4;
-    return left >= 2 ? 2 : 1;
+    const bool small = (long long)h->nx * h->ny <= 150000;
+    if (small && left >= 4) return 4;
+    return left >= 2 && (small || two_steps_pay(h)) ? 2 : 1;
 }
 
 // K steps from fin to fout; g32 and g_step: the first step's force and the
