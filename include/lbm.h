@@ -239,6 +239,12 @@ lbm_status lbm_get_launch(const lbm_handle *h, int *block_x, int *nodes_per_thre
  * falls back for what is left over), else 1.  lbm_set_launch and
  * lbm_set_launch_layout set 1; lbm_autotune keeps what it measures faster. */
 lbm_status lbm_get_launch_steps(const lbm_handle *h, int *steps);
+/* Take one step per launch (1), or several: 4 up to 150,000 nodes and 2 above,
+ * on a D2Q9 handle in FP32, FP16 or BF16 storage wider than 4 nodes along each
+ * axis and below 4 GB of state (LBM_ERR_ARG otherwise).  Restores a choice of
+ * lbm_autotune; the launch shape stays.  Drops the captured step graphs;
+ * synchronises the handle's stream. */
+lbm_status lbm_set_launch_steps(lbm_handle *h, int steps);
 /* The two vector widths (nodes per thread; equal when only one is built) of
  * LBM_LAYOUT_VECTOR for a lattice and storage (outputs nullable). */
 lbm_status lbm_launch_widths(int lattice, int storage, int *lo, int *hi);

@@ -84,6 +84,7 @@ def library():
     L.lbm_set_launch_layout.argtypes = [H, C.c_int, C.c_int, C.c_int]
     L.lbm_get_launch.argtypes = [H, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int)]
     L.lbm_get_launch_steps.argtypes = [H, C.POINTER(C.c_int)]
+    L.lbm_set_launch_steps.argtypes = [H, C.c_int]
     L.lbm_launch_widths.argtypes = [C.c_int, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_int)]
     L.lbm_force_resolution.argtypes = [H, dp]
     L.lbm_alu_peak.argtypes = [C.c_int, C.c_int64, dp, dp]
@@ -130,7 +131,7 @@ def library():
               "lbm_check_device",
               "lbm_set_force", "lbm_set_force_schedule", "lbm_set_force_scale_schedule", "lbm_get_populations", "lbm_set_populations", "lbm_get_state",
               "lbm_set_state", "lbm_info", "lbm_set_launch", "lbm_set_launch_layout", "lbm_get_launch",
-              "lbm_get_launch_steps",
+              "lbm_get_launch_steps", "lbm_set_launch_steps",
               "lbm_launch_widths", "lbm_force_resolution", "lbm_alu_peak", "lbm_autotune", "lbm_check_noalloc", "lbm_split_schedule", "lbm_split_create",
               "lbm_split_step", "lbm_split_check_device", "lbm_split_moments", "lbm_split_get_state",
               "lbm_split_get_populations", "lbm_split_set_launch_layout",
@@ -310,6 +311,10 @@ def lbm_get_launch_steps(h):
     return k.value
 
 
+def lbm_set_launch_steps(h, steps):
+    _check(library().lbm_set_launch_steps(h, int(steps)), h)
+
+
 def lbm_launch_widths(lattice, storage):
     lo, hi = C.c_int(), C.c_int()
     _check(library().lbm_launch_widths(_enum("lattice", lattice), _enum("storage", storage), C.byref(lo),
@@ -460,6 +465,10 @@ class Lattice:
         """Time steps per kernel launch of a long step() (see lbm_get_launch_steps)."""
         return lbm_get_launch_steps(self.h)
 
+    def set_launch_steps(self, steps):
+        """One step per launch (1) or several (see lbm_set_launch_steps)."""
+        lbm_set_launch_steps(self.h, steps)
+
     def force_resolution(self):
         """Speed above which one step of the force rounds away in the storage
         format (see lbm_force_resolution); inf without a force."""
@@ -472,22 +481,23 @@ class Lattice:
     def autotune(self, trials=20, cache=None):
         """Pick the fastest launch shape (see lbm_autotune).  With a cache path,
         reuse a stored choice for the same problem signature or store the new
-        one (JSON keyed by lattice, collision, storage, sizes, mask, device)."""
+        one (JSON keyed by lattice, collision, storage, sizes, mask, device).
+        An entry without the steps per launch was measured before there were
+        several: it is reused only on a handle that takes one."""
         key = None
         if cache:
             from . import autotune as A
             key = A.signature(self)
             hit = A.lookup(cache, key)
-            if hit:
-                # the shape a new handle starts with stays as it is: setting
-                # it would give up several steps per launch
-                if tuple(hit["launch"]) != self.launch():
-                    self.set_launch(*hit["launch"])
+            if hit and ("steps" in hit or self.launch_steps() == 1):
+                self.set_launch(*hit["launch"])
+                if hit.get("steps", 1) > 1:
+                    self.set_launch_steps(hit["steps"])
                 return tuple(hit["launch"]) + (hit["ms"],)
         bx, npt, ms = lbm_autotune(self.h, trials)
         if cache:
             from . import autotune as A
-            A.store(cache, key, self.launch(), ms)
+            A.store(cache, key, self.launch(), ms, self.launch_steps())
         return bx, npt, ms
 
     def close(self):

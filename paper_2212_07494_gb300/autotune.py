@@ -1,4 +1,4 @@
-"""JSON cache of launch shapes chosen by lbm_autotune, keyed by the problem
+"""JSON cache of launch shapes and steps per launch chosen by lbm_autotune, keyed by the problem
 signature (lattice, collision, storage, sizes, obstacle mask) and the device
 name, so a shape measured once is reused by later runs of the same problem."""
 from __future__ import annotations
@@ -31,7 +31,7 @@ def lookup(path: str, key: str):
         return None
 
 
-def store(path: str, key: str, launch, ms: float) -> None:
+def store(path: str, key: str, launch, ms: float, steps: int | None = None) -> None:
     data = {}
     try:
         with open(path) as f:
@@ -39,6 +39,8 @@ def store(path: str, key: str, launch, ms: float) -> None:
     except (OSError, ValueError):
         pass
     data[key] = {"launch": list(launch), "ms": ms}
+    if steps is not None:
+        data[key]["steps"] = steps
     d = os.path.dirname(os.path.abspath(path))
     os.makedirs(d, exist_ok=True)
     fd, tmp = tempfile.mkstemp(dir=d)

@@ -119,6 +119,10 @@ cudaError_t launch_finalize(const double *partials, int nblocks, double *out, cu
 void set_thread_error(const char *msg) { g_thread_err = msg; }
 }  // namespace lbm
 
+// several steps per launch: never, where they were measured faster
+// (two_steps_pay), wherever k_step_tile applies
+enum { FUSE_OFF = 0, FUSE_RULE = 1, FUSE_ON = 2 };
+
 struct lbm_handle {
     int lattice = 0, collision = 0, storage = 0;
     int D = 2, Q = 9;
@@ -158,7 +162,7 @@ struct lbm_handle {
     double *gring_dev = nullptr;
     float *gring32_dev = nullptr;
     int graph_steps = 0;
-    bool fuse = false;           // several steps per launch (k_step_tile)
+    int fuse = FUSE_OFF;         // several steps per launch (k_step_tile)
     bool hold_fuse = false;      // not in the current call (a caller's stream capture)
     int64_t step = 0;
     void *(*alloc)(size_t, void *) = nullptr;
@@ -321,11 +325,16 @@ bool two_steps_pay(const lbm_handle *h) {
 // the margins' extra collisions are hidden.  From about 1.5e5 nodes on the
 // collisions fill the chip and two steps are faster (F32, us per step, four
 // against two: 400 x 300 1.82 / 1.95, 512^2 2.95 / 2.82, 1024^2 9.3 / 7.4).
+int tile_steps_of(const lbm_handle *h) {
+    if (!tile_ok(h) || (h->gs_dev && !h->gring_dev)) return 1;
+    return (long long)h->nx * h->ny <= 150000 ? 4 : 2;
+}
 int fused_steps(const lbm_handle *h, int64_t left) {
-    if (!h->fuse || h->hold_fuse || !tile_ok(h) || (h->gs_dev && !h->gring_dev)) return 1;
-    const bool small = (long long)h->nx * h->ny <= 150000;
-    if (small && left >= 4) return 4;
-    return left >= 2 && (small || two_steps_pay(h)) ? 2 : 1;
+    if (h->fuse == FUSE_OFF || h->hold_fuse) return 1;
+    const int k = tile_steps_of(h);
+    if (k == 4 && left >= 4) return 4;
+    if (k == 2 && h->fuse == FUSE_RULE && !two_steps_pay(h)) return 1;
+    return k > 1 && left >= 2 ? 2 : 1;
 }
 
 // K steps from fin to fout; g32 and g_step: the first step's force and the
@@ -728,7 +737,7 @@ lbm_status lbm_create(const lbm_desc *d, lbm_handle **out) {
         h->cfg.bdx = 128;
     }
     h->graph_steps = 64;
-    h->fuse = true;   // where k_step_tile applies (tile_ok)
+    h->fuse = FUSE_RULE;
 
     lbm_status st;
     if (d->stream) {
@@ -1070,7 +1079,7 @@ lbm_status lbm_set_launch_layout(lbm_handle *h, int block_x, int nodes_per_threa
     }
     LBM_CUDA(h, cudaStreamSynchronize(h->stream));
     h->cfg = c;
-    h->fuse = false;
+    h->fuse = FUSE_OFF;
     drop_graphs(h);
     return LBM_OK;
 }
@@ -1078,6 +1087,16 @@ lbm_status lbm_set_launch_layout(lbm_handle *h, int block_x, int nodes_per_threa
 lbm_status lbm_get_launch_steps(const lbm_handle *h, int *steps) {
     if (!h || !steps) return fail(nullptr, LBM_ERR_ARG, "NULL argument");
     *steps = fused_steps(h, 64);
+    return LBM_OK;
+}
+
+lbm_status lbm_set_launch_steps(lbm_handle *h, int steps) {
+    if (!h) return fail(nullptr, LBM_ERR_ARG, "handle is NULL");
+    if (steps != 1 && steps != tile_steps_of(h))
+        return fail(h, LBM_ERR_ARG, "steps must be 1, or 4 or 2 as the domain's size gives where several steps apply");
+    LBM_CUDA(h, cudaStreamSynchronize(h->stream));
+    h->fuse = steps > 1 ? FUSE_ON : FUSE_OFF;
+    drop_graphs(h);
     return LBM_OK;
 }
 
@@ -1123,8 +1142,7 @@ lbm_status lbm_autotune(lbm_handle *h, int trials, int *block_x, int *nodes_per_
     double best = 1e300;
     StepCfg best_cfg = h->cfg;
     // several steps per launch first (where it applies), then the shapes
-    h->fuse = true;
-    const int K = fused_steps(h, 64);
+    const int K = tile_steps_of(h);
     bool best_fused = false;
     for (int v = K > 1 ? -1 : 0; v < (int)shapes.size(); ++v) {
         const bool fused = v < 0;
@@ -1154,7 +1172,9 @@ lbm_status lbm_autotune(lbm_handle *h, int trials, int *block_x, int *nodes_per_
     cudaEventDestroy(e1);
     if (e != cudaSuccess) return cuda_fail(h, e, "autotune");
     drop_graphs(h);
-    if (!best_fused) {
+    if (best_fused) {
+        h->fuse = FUSE_ON;
+    } else {
         lbm_status st = lbm_set_launch_layout(h, best_cfg.bdx, best_cfg.npt,
                                               best_cfg.vec ? LBM_LAYOUT_VECTOR : LBM_LAYOUT_STRIDED);
         if (st != LBM_OK) return st;
