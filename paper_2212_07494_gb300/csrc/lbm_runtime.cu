@@ -1033,9 +1033,6 @@ lbm_status lbm_set_populations(lbm_handle *h, const double *f) {
     cudaError_t e = cudaMemcpyAsync(tmp, f, n * sizeof(double), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = L.put_pops(h->storage, h->kp, tmp, spare, h->stream);
     if (e == cudaSuccess) e = L.unstream(h->storage, h->mask, h->kp, spare, h->buf[h->cur], h->stream);
-    // the steps never write solid nodes: clear what the import left there, so
-    // that the raw state does not depend on which buffer a run ends in
-    if (e == cudaSuccess && h->mask) e = cudaMemsetAsync(spare, 0, h->state_bytes, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     dev_free(h, tmp);
     if (e != cudaSuccess) return cuda_fail(h, e, "population import");
