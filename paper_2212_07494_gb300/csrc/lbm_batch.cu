@@ -1108,7 +1108,7 @@ lbm_status lbm_batch_create(const lbm_desc *descs, int n, lbm_batch **out) {
     if (e == cudaSuccess && solid_bytes)
         e = cudaMemsetAsync(b->links, 0, (size_t)solid_bytes * sizeof(unsigned), b->stream);
     for (int c = 0; c < n && e == cudaSuccess; ++c)
-        if (descs[c].solid) e = launchers_d2q9().links(b->kp[c], b->links + b->ch[c].solid_off, nullptr, b->stream);
+        if (descs[c].solid) e = launchers_d2q9().links(b->kp[c], b->links + b->ch[c].solid_off, b->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->g32_dev, g32.data(), g32.size() * 4, cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->fa, 0, (size_t)off * eb, b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->fb, 0, (size_t)off * eb, b->stream);

@@ -143,8 +143,8 @@ struct Launchers {
     cudaError_t (*get_pops)(int st, bool mask, const KParams &p, const void *state, double *out,
                             cudaStream_t s);
     cudaError_t (*put_pops)(int st, const KParams &p, const double *in, void *target, cudaStream_t s);
-    // obstacle links of every node from p.solid (KParams.links); *linked (device, may be null) += nodes with any
-    cudaError_t (*links)(const KParams &p, unsigned *links, unsigned *linked, cudaStream_t s);
+    // obstacle links of every node from p.solid (KParams.links)
+    cudaError_t (*links)(const KParams &p, unsigned *links, cudaStream_t s);
 };
 
 const Launchers &launchers_d2q9();

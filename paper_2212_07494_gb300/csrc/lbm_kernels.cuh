@@ -333,28 +333,24 @@ __global__ void k_unstream(const KParams p, const typename Store<ST>::T *__restr
 }
 
 // Obstacle links of every node a pull can be asked for (a slab's halo layers
-// excluded) from the mask.  linked: number of nodes with any link or solid.
+// excluded) from the mask.
 template <int L>
-__global__ void k_links(const KParams p, unsigned *__restrict__ links, unsigned *linked) {
+__global__ void k_links(const KParams p, unsigned *__restrict__ links) {
     const int y = blockIdx.y + (p.halo_ax == 1), z = blockIdx.z + (p.halo_ax == 2);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned b = 0u;
-    if (x < p.nx) {
-        const long long own = node_index(p, x, y, z);
-        NodeNbr nb;
-        node_nbr(p, x, y, z, nb);
-        b = p.solid[own] ? 1u : 0u;
+    if (x >= p.nx) return;
+    const long long own = node_index(p, x, y, z);
+    NodeNbr nb;
+    node_nbr(p, x, y, z, nb);
+    unsigned b = p.solid[own] ? 1u : 0u;
 #pragma unroll
-        for (int i = 1; i < Lat<L>::Q; ++i) {
-            const int kx = Lat<L>::cx(i) + 1, ky = Lat<L>::cy(i) + 1, kz = Lat<L>::cz(i) + 1;
-            const bool wall = nb.xw[kx] || nb.yw[ky] || (Lat<L>::D == 3 && nb.zw[kz]);
-            const long long src = node_index(p, nb.xs[kx], nb.ys[ky], Lat<L>::D == 3 ? nb.zs[kz] : z);
-            if (!wall && p.solid[src] != 0) b |= 1u << i;
-        }
-        links[own] = b;
+    for (int i = 1; i < Lat<L>::Q; ++i) {
+        const int kx = Lat<L>::cx(i) + 1, ky = Lat<L>::cy(i) + 1, kz = Lat<L>::cz(i) + 1;
+        const bool wall = nb.xw[kx] || nb.yw[ky] || (Lat<L>::D == 3 && nb.zw[kz]);
+        const long long src = node_index(p, nb.xs[kx], nb.ys[ky], Lat<L>::D == 3 ? nb.zs[kz] : z);
+        if (!wall && p.solid[src] != 0) b |= 1u << i;
     }
-    const unsigned m = __ballot_sync(0xffffffffu, b != 0u);
-    if (linked && m != 0u && (threadIdx.x & 31) == 0) atomicAdd(linked, (unsigned)__popc(m));
+    links[own] = b;
 }
 
 // Pre-collision populations fbar = w + delta in FP64, unpadded [Q][N]
@@ -525,8 +521,8 @@ template <int L> struct Dispatch {
         return cudaErrorInvalidValue;
     }
 
-    static cudaError_t links(const KParams &p, unsigned *out, unsigned *linked, cudaStream_t s) {
-        k_links<L><<<step_grid(p, 128, 1), 128, 0, s>>>(p, out, linked);
+    static cudaError_t links(const KParams &p, unsigned *out, cudaStream_t s) {
+        k_links<L><<<step_grid(p, 128, 1), 128, 0, s>>>(p, out);
         return cudaGetLastError();
     }
 

@@ -609,7 +609,7 @@ lbm_status handle_make_slab(lbm_handle *h, int ax, int g0, int gn) {
     h->kp.hgn = gn;
     drop_graphs(h);
     if (h->mask)
-        LBM_CUDA(h, launchers_for(h->lattice).links(h->kp, h->links_dev, nullptr, h->stream));
+        LBM_CUDA(h, launchers_for(h->lattice).links(h->kp, h->links_dev, h->stream));
     return LBM_OK;
 }
 
@@ -813,7 +813,7 @@ lbm_status lbm_create(const lbm_desc *d, lbm_handle **out) {
             return fail(nullptr, st, m);
         }
         e = cudaMemsetAsync(h->links_dev, 0, (size_t)plane * sizeof(unsigned), h->stream);
-        if (e == cudaSuccess) e = launchers_for(h->lattice).links(kp, h->links_dev, nullptr, h->stream);
+        if (e == cudaSuccess) e = launchers_for(h->lattice).links(kp, h->links_dev, h->stream);
         if (e != cudaSuccess) {
             lbm_status s2 = cuda_fail(nullptr, e, "obstacle links");
             lbm_destroy(h);

@@ -1858,7 +1858,6 @@ bool conv_col(lbm_unet *u, const ConvArgs &a, lbm_status *st) {
 
 template <int BK> lbm_status launch_conv_n(lbm_unet *u, const ConvArgs &a, long long M) {
     lbm_status st = LBM_OK;
-    if (a.cout <= 16) return launch_tma<BK, 16>(u, a, &st) ? st : launch_tc<BK, 16>(u, a, M);
     if (a.cout <= 32) return launch_tma<BK, 32>(u, a, &st) ? st : launch_tc<BK, 32>(u, a, M);
     if (a.cout <= 64) return launch_tma<BK, 64>(u, a, &st) ? st : launch_tc<BK, 64>(u, a, M);
     return launch_tma<BK, 128>(u, a, &st) ? st : launch_tc<BK, 128>(u, a, M);
