@@ -317,6 +317,13 @@ def make_lattice(P, wl, spec, st, coll, tau_bulk=0.0, torch_stream=None, host_in
                      rho0=rho0, u0=u0, torch_stream=torch_stream, tau_bulk=tau_bulk)
 
 
+def step_launches(n, K):
+    """Step kernels of one step(n) call with K steps per launch: what is left over goes in smaller launches, and one
+    launch is halved where launches and steps would differ by an odd number."""
+    m = n // K + (n % K) // 2 + (n % K) % 2 if K > 1 else n
+    return m + (n - m) % 2
+
+
 def run_gpu(args, ws, rank, local):
     import torch
 
@@ -415,12 +422,8 @@ def run_gpu(args, ws, rank, local):
     traffic = (traffic_per_launch(N, coll)
                if st == "F32" and not args.tau_bulk and spec["lattice"] == "D2Q9" and K == 1 else None)
     clocks = sampler.summary()
-    # step kernels (runs of n steps: K per launch, what is left over in smaller ones, one more where the launches would
-    # differ from the steps by an odd number), and the moments and finalize kernels per check
-    launches = 2 * k
-    for _, _, n in chunk_ev:
-        m = n // K + (n % K) // 2 + (n % K) % 2 if K > 1 else n
-        launches += m + (n - m) % 2
+    # step kernels, and the moments and finalize kernels per check
+    launches = sum(step_launches(n, K) for _, _, n in chunk_ev) + 2 * k
 
     e2e = None
     if not args.no_e2e:
@@ -994,6 +997,7 @@ def run_womersley(args, ws, rank, local):
     ua = womersley_analytic(y, t_end, A, om, nu, ny / 2)
     err = float(np.abs(u[0, 0, :, 0] - ua).max() / (A / om))
     f_sched = lat.populations()
+    K = lat.launch_steps()
     lat.close()
     # the same steps with a host call per step
     ref = P.Lattice("D2Q9", "SMRT", (nx, ny, 1), tau, "F32", (1, 0, 1), g=tab[0])
@@ -1017,7 +1021,8 @@ def run_womersley(args, ws, rank, local):
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": None, "note": "10,000 nodes per step: launch latency bounds it, not HBM",
                          "peak_source": f"{peak_kind} hbm_gbs (copy)"},
-            "gpu_launches": 2 * steps + steps // 64,   # k_step and the force update per step, a counter advance per 64
+            # the step kernels, and per 64 steps the forces laid out at once and the counter's advance
+            "gpu_launches": step_launches(steps, K) + 2 * -(-steps // 64), "steps_per_launch": K,
             "clocks": sampler.summary(),
             "per_step_set_force": {"seconds": host_s, "steps": t_end, "mlups": N * t_end / host_s / 1e6,
                                    "us_per_step": host_s / t_end * 1e6},

@@ -12,6 +12,12 @@
 // scheduler, 64 clocks an instruction) 7.65 and 4.26.  Against a long double
 // reference one collision is closer than the shared form's (relative error
 // 1.28e-16 against 1.72e-16 for SMRT, 1.49e-16 against 1.86e-16 for BGK).
+// Runs of the two SMRT forms drift apart by more than that, 3.7e-13 after 600
+// steps of a 50 x 200 channel: in double the line weights 1/6 + 2/3 + 1/6 add
+// up to 1 - 5.6e-17, so the shared reconstruction, which multiplies by them,
+// loses that share of mass and momentum per line and step (mean momentum lost
+// per collision at j = 0.05: 7.6e-18 +- 0.1e-18; here 0 +- 0.07e-18), as does
+// any reference written with those three constants.
 #pragma once
 #include "lbm_device.cuh"
 

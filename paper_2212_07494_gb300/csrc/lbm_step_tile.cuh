@@ -18,10 +18,11 @@
 // sources node by node.
 //
 // What bounds it: on a large FP32 domain memory (36 bytes per node and step
-// with K = 2: 90 us for 4096^2) and the packed FP32 pipe (about 150 f32x2
-// instructions per pair and step at half rate, 67 us) together; 2-byte
-// storage the packed FP32 pipe; a small domain the latency of a launch and of
-// a step's dependent instructions.  us per step, one step per launch and
+// with K = 2: 90 us for 4096^2) and instructions together (2048^2: DRAM 56 %,
+// FMA pipe 62 %, issue 66 % busy; 338 warp instructions per pair and step, 177
+// of them on the FMA pipe, margins included); 2-byte storage the instructions
+// (FMA pipe 65 %, issue 68 %, DRAM 26 %); a small domain the latency of a
+// launch and of a step's dependent instructions.  us per step, one step per launch and
 // this kernel, residual and moments included: 4096^2 FP32 183.0 and 114.0
 // (1.605x), 4096^2 FP16 101.0 and 99.8, 1001 x 517 with walls 8.90 and 5.21,
 // 256 x 128 with obstacles 3.19 and 1.41.

@@ -5,8 +5,10 @@
 // kernels.
 //
 // Activations are NHWC bfloat16; every contraction accumulates in FP32 on the
-// tensor cores (mma.sync m16n8k16 BF16, operands staged by cp.async and read
-// with ldmatrix).  Convolutions are implicit GEMMs:
+// 5th-generation tensor cores (tcgen05, operands by TMA, accumulators in TMEM)
+// where the shape allows, else on mma.sync m16n8k16.  Convolutions are implicit
+// GEMMs (k_conv_col up to 128 input channels, k_conv_tma above, k_conv_ws and
+// k_conv for shapes neither takes):
 //   forward      y[p][co]  = sum_{tap,ci} x[p+tap][ci] W[co][tap][ci]
 //   input grad   dx[p][ci] = sum_{tap,co} dz[p-tap][co] W[co][tap][ci]
 //                (the same kernel with the flipped, transposed weights)
