@@ -179,7 +179,6 @@ struct KParams {
     // index of layer 1 and hgn the global extent, which place the domain's
     // walls on that axis.
     int halo_ax, hg0, hgn;
-    // per population i, relative to a node's element index:
     // per population i, relative to the element index of a node's x - c_x
     // (the node itself, or its neighbour along x, wrapped on a periodic x):
     long long doff[27];            // i*plane - (cy*nxp + cz*nxp*ny): pull source

@@ -37,9 +37,24 @@ __device__ __noinline__ void step_node_alone(const KParams &p, const typename St
     for (int i = 0; i < Lat<L>::Q; ++i) Store<ST>::st(dst + p.poff[i], G[gpos<L>(i)]);
 }
 
+// k_step's parameters.  In FP64 the offset table starts on a 16-byte boundary
+// here, 8 bytes further than KParams alone puts it (us per step, without and
+// with: 64 x 32 BGK 4.27 and 4.24, 50 x 200 SMRT with a schedule 5.00 and 4.95);
+// the kernels in FP32 arithmetic keep theirs (D3Q19 BF16 256^2 x 200 208 and
+// 209).
+template <int ST> struct StepArg {
+    KParams p;
+};
+template <> struct StepArg<ST_F64> {
+    long long lead;
+    KParams p;
+};
+static_assert((offsetof(StepArg<ST_F64>, p) + offsetof(KParams, doff)) % 16 == 0, "the FP64 offset table's alignment");
+
 template <int L, int COLL, int ST, bool MASK, int NPT>
-__global__ void __launch_bounds__(256, step_min_blocks<ST>()) k_step(const __grid_constant__ KParams p, const typename Store<ST>::T *__restrict__ fin,
+__global__ void __launch_bounds__(256, step_min_blocks<ST>()) k_step(const __grid_constant__ StepArg<ST> arg, const typename Store<ST>::T *__restrict__ fin,
                                               typename Store<ST>::T *__restrict__ fout) {
+    const KParams &p = arg.p;
     typedef typename Store<ST>::R R;
     constexpr int NG = Grid<Lat<L>::D>::N;
     const int y = blockIdx.y + (p.halo_ax == 1), z = blockIdx.z + (p.halo_ax == 2);
@@ -393,8 +408,10 @@ template <int L> struct Dispatch {
     template <int COLL, int ST, bool MASK, int NPT>
     static cudaError_t step_t(StepCfg cfg, const KParams &p, const void *fin, void *fout, cudaStream_t s) {
         typedef typename Store<ST>::T T;
+        StepArg<ST> arg{};
+        arg.p = p;
         k_step<L, COLL, ST, MASK, NPT><<<step_grid(p, cfg.bdx, NPT), cfg.bdx, 0, s>>>(
-            p, (const T *)fin, (T *)fout);
+            arg, (const T *)fin, (T *)fout);
         return cudaGetLastError();
     }
     template <int COLL, int ST, bool MASK>
