@@ -18,10 +18,10 @@
 // Population data written during the kernel by other CTAs is read through L2
 // (ld.global.cg), never through the non-coherent read-only path.
 //
-// In FP32, steps without a residual check are taken two at a time: a tile is
-// then a run of kFuseX x kFuseY node tiles of the channel, each advanced by
-// two steps in shared memory (tile_steps of lbm_step_tile.cuh, bit for bit
-// the two single steps).  That halves the claims, the fences and the memory
+// In FP32, with kFuseMinK steps or more from check to check, the steps without
+// one are taken two at a time: a tile is then a run of kFuseX x kFuseY node
+// tiles of the channel, each advanced by two steps in shared memory (tile_steps
+// of lbm_step_tile.cuh, bit for bit the two single steps).  That halves the claims, the fences and the memory
 // traffic per step.  A channel's state moves to the other arena with every
 // claim's worth of steps, whether one or two (BatchCtl.flips).
 #include <cuda_runtime.h>
@@ -63,12 +63,13 @@ struct BatchChan {
 constexpr int kTileBits = 13;
 constexpr unsigned long long kTileMask = (1ull << kTileBits) - 1;
 constexpr int kMaxTiles = 4096;
-__host__ __device__ inline unsigned long long claim_word(long long step, int tiles) {
-    return ((unsigned long long)step << (2 * kTileBits)) | ((unsigned long long)tiles << kTileBits);
+// a channel's next step, the parity of its flips (the arena its state is in) and the step's tiles
+__host__ __device__ inline unsigned long long claim_word(long long step, int flips, int tiles) {
+    return ((unsigned long long)(2 * step + (flips & 1)) << (2 * kTileBits)) | ((unsigned long long)tiles << kTileBits);
 }
 
 struct BatchCtl {
-    unsigned long long claim;  // claim_word(step, tiles) + next tile index
+    unsigned long long claim;  // claim_word(step, flips, tiles) + next tile index
     unsigned int done;         // tiles finished in the current step
     int active;
     long long steps;           // steps completed
@@ -106,6 +107,12 @@ struct BatchRun {
 // blocks of 128 threads: 32 x 16 51, 30 x 14 56, 62 x 14 66, three steps of
 // 32 x 8 69; one step at a time, in row bands, 87.
 constexpr int kFuseSteps = 2, kFuseX = 32, kFuseY = 16;
+// The shortest check interval that takes pairs of steps.  A check step and an
+// odd step out are single, and single steps cost more in the kernel that can
+// take pairs: ms for 250 steps of 48 channels without and with pairs, K = 4:
+// SMRT 8.2 / 8.9, SMRT_FNEQ 7.3 / 9.7; K = 6: 7.9 / 7.4, 6.9 / 8.2; K = 8: 7.9 /
+// 6.5, 6.9 / 7.3; K = 9: 7.9 / 5.2, 6.9 / 6.1; K = 20: 8.1 / 4.5, 6.8 / 5.0.
+constexpr int kFuseMinK = 9;
 
 // whether a channel that started its run at step `start` takes kFuseSteps
 // steps at once from `step` on: none of them checks the residual (the steps
@@ -283,13 +290,14 @@ __device__ __noinline__ void batch_fused(const BatchRun &r, int c, const float *
 }
 
 // batch storage is FP32 or FP64 (loads through L2: ld.global.cg).  The
-// launch bounds cap the kernel at 64 registers (no spills in FP32), so 8
-// blocks of 128 threads share an SM instead of 6.
-template <int COLL, int ST>
+// launch bounds cap the kernel at 64 registers, so 8 blocks of 128 threads
+// share an SM instead of 6.  FUSE: the instance that can take pairs of steps
+// (its call makes the single step spill more and its tiles take shared memory).
+template <int COLL, int ST, bool FUSE>
 __global__ void __launch_bounds__(256, 4) k_batch(const __grid_constant__ BatchRun r) {
     typedef typename Store<ST>::T T;
     typedef typename Store<ST>::R R;
-    __shared__ int s_c, s_tile, s_tiles, s_quit, s_flips;
+    __shared__ int s_c, s_tile, s_tiles, s_quit, s_odd;
     __shared__ long long s_step;
     long long empty = 0;
     unsigned long long seen = 0;
@@ -319,10 +327,12 @@ __global__ void __launch_bounds__(256, 4) k_batch(const __grid_constant__ BatchR
                     }
                     unsigned m = __ballot_sync(0xffffffffu, ok);
                     while (m != 0u) {
-                        // CTAs start at different channels of the word: with
-                        // the lowest one first, all of them added to the same
-                        // few claim words and most came too late
-                        const int pick = (int)__fns(m, 0, 1 + (int)(blockIdx.x % (unsigned)__popc(m)));
+                        // with pairs of steps, CTAs start at different channels
+                        // of the word: with the lowest one first, all of them
+                        // added to the same few claim words and most came too late
+                        const bool mine = FUSE && ((m >> lane) & 1u) != 0u &&
+                                          __popc(m & ((1u << lane) - 1u)) == (int)(blockIdx.x % (unsigned)__popc(m));
+                        const int pick = __ffs(FUSE ? __ballot_sync(0xffffffffu, mine) : m) - 1;
                         m &= ~(1u << pick);
                         unsigned long long w2 = 0ull;
                         if (lane == pick) w2 = atomicAdd(&r.ctl[c].claim, 1ull);
@@ -340,7 +350,8 @@ __global__ void __launch_bounds__(256, 4) k_batch(const __grid_constant__ BatchR
             }
             if (lane == 0) {
                 s_c = fc;
-                s_step = fs;
+                s_step = fs >> 1;
+                s_odd = (int)(fs & 1);
                 s_tile = ft;
                 s_tiles = fn;
                 s_quit = 0;
@@ -362,8 +373,6 @@ __global__ void __launch_bounds__(256, 4) k_batch(const __grid_constant__ BatchR
                     empty = 0;
                 }
                 __threadfence();
-                // written before the claim word that opened these tiles
-                if (fc >= 0) s_flips = vload(&r.ctl[fc].flips);
             }
         }
         __syncthreads();
@@ -375,12 +384,12 @@ __global__ void __launch_bounds__(256, 4) k_batch(const __grid_constant__ BatchR
             const int tile = s_tile;
             const int ntiles = s_tiles;
             const int rows = (C.ny + ntiles - 1) / ntiles;
-            const int flips = s_flips;
-            const T *fin = (const T *)((flips & 1) ? r.fb : r.fa) + C.off;
-            T *fout = (T *)((flips & 1) ? r.fa : r.fb) + C.off;
+            const int odd = s_odd;
+            const T *fin = (const T *)(odd ? r.fb : r.fa) + C.off;
+            T *fout = (T *)(odd ? r.fa : r.fb) + C.off;
             const long long start = r.ctl[c].start;
             const bool check = ((step - start) % r.K) == 0;
-            const bool fused = ST == ST_F32 && fused_at(C, step, start, r.K, r.max_steps);
+            const bool fused = FUSE && fused_at(C, step, start, r.K, r.max_steps);
             const int y0 = tile * rows;
             const int y1 = min(y0 + rows, C.ny);
             const int nn = !fused && y1 > y0 ? (y1 - y0) * C.nx : 0;  // the last tiles may be empty
@@ -390,7 +399,7 @@ __global__ void __launch_bounds__(256, 4) k_batch(const __grid_constant__ BatchR
             const R om2 = R(C.om2), om3 = R(C.om3), om4 = R(C.om4), gx = R(C.gx), gy = R(C.gy);
             const bool trim = C.om3 == 1.0 && C.om4 == 1.0;
             double v[2] = {0.0, 0.0};
-            if constexpr (ST == ST_F32) {
+            if constexpr (FUSE) {
                 if (fused) {
                     if constexpr (COLL == SMRT) {
                         if (trim) batch_fused<SMRT_TRIM>(r, c, fin, fout, tile, ntiles);
@@ -528,7 +537,7 @@ __global__ void __launch_bounds__(256, 4) k_batch(const __grid_constant__ BatchR
                         status = r.tol >= 0.0 ? (int)LBM_NOT_CONVERGED : (int)LBM_OK;
                     }
                     r.ctl[c].steps = done_steps;
-                    r.ctl[c].flips = flips + 1;
+                    r.ctl[c].flips = vload(&r.ctl[c].flips) + 1;
                     atomicExch(&r.ctl[c].done, 0u);
                     // the tail: few channels left, each would take a whole
                     // scheduling round per step here; they leave at this step
@@ -543,12 +552,12 @@ __global__ void __launch_bounds__(256, 4) k_batch(const __grid_constant__ BatchR
                         atomicAdd((unsigned long long *)r.active_nodes, (unsigned long long)(-(long long)C.nx * C.ny));
                         atomicSub(r.active_count, 1);
                     } else {
-                        const bool next_fused = ST == ST_F32 && fused_at(C, done_steps, start, r.K, r.max_steps);
+                        const bool next_fused = FUSE && fused_at(C, done_steps, start, r.K, r.max_steps);
                         const long long active = vload(r.active_nodes);
                         const int nt = next_fused ? fused_tiles_for(C, active, r)
                                                   : tiles_for(C.nx, C.ny, active, r.grid, r.tile_min, r.tile_max);
                         __threadfence();
-                        atomicExch(&r.ctl[c].claim, claim_word(done_steps, nt));
+                        atomicExch(&r.ctl[c].claim, claim_word(done_steps, odd + 1, nt));
                     }
                     atomicAdd(r.progress, 1ull);
                 }
@@ -564,7 +573,7 @@ __global__ void k_batch_reset(BatchRun r, long long total_nodes) {
     if (c < r.n) {
         BatchCtl *ctl = r.ctl;
         const long long s = ctl[c].steps;
-        ctl[c].claim = claim_word(s, tiles_for(r.ch[c].nx, r.ch[c].ny, total_nodes, r.grid, r.tile_min, r.tile_max));
+        ctl[c].claim = claim_word(s, ctl[c].flips, tiles_for(r.ch[c].nx, r.ch[c].ny, total_nodes, r.grid, r.tile_min, r.tile_max));
         ctl[c].done = 0u;
         ctl[c].active = 1;
         ctl[c].start = s;
@@ -677,12 +686,16 @@ typedef void (*BatchKernel)(const BatchRun);
 
 // SMRT with every channel at tau_3 = tau_4 = 1 takes the kernel built for the
 // trimmed collision alone
-BatchKernel batch_kernel(int coll, int st, bool all_trim) {
-    if (coll == LBM_SMRT && all_trim) return st == LBM_F64 ? k_batch<SMRT_TRIM, ST_F64> : k_batch<SMRT_TRIM, ST_F32>;
-    if (coll == LBM_SMRT) return st == LBM_F64 ? k_batch<SMRT, ST_F64> : k_batch<SMRT, ST_F32>;
-    if (coll == LBM_SMRT_FNEQ) return st == LBM_F64 ? k_batch<SMRT_FNEQ, ST_F64> : k_batch<SMRT_FNEQ, ST_F32>;
-    if (coll == LBM_MRT_RAW) return st == LBM_F64 ? k_batch<MRT_RAW, ST_F64> : k_batch<MRT_RAW, ST_F32>;
-    return st == LBM_F64 ? k_batch<BGK, ST_F64> : k_batch<BGK, ST_F32>;
+template <int ST, bool FUSE> BatchKernel batch_kernel_of(int coll, bool all_trim) {
+    if (coll == LBM_SMRT && all_trim) return k_batch<SMRT_TRIM, ST, FUSE>;
+    if (coll == LBM_SMRT) return k_batch<SMRT, ST, FUSE>;
+    if (coll == LBM_SMRT_FNEQ) return k_batch<SMRT_FNEQ, ST, FUSE>;
+    if (coll == LBM_MRT_RAW) return k_batch<MRT_RAW, ST, FUSE>;
+    return k_batch<BGK, ST, FUSE>;
+}
+BatchKernel batch_kernel(int coll, int st, bool fuse, bool all_trim) {
+    if (st == LBM_F64) return batch_kernel_of<ST_F64, false>(coll, all_trim);
+    return fuse ? batch_kernel_of<ST_F32, true>(coll, all_trim) : batch_kernel_of<ST_F32, false>(coll, all_trim);
 }
 
 bool all_trim(const lbm_batch *b) {
@@ -693,11 +706,12 @@ bool all_trim(const lbm_batch *b) {
 
 // one run: reset + persistent kernel, captured in a graph and launched once
 lbm_status batch_run(lbm_batch *b, double tol, int K, int64_t max_steps) {
-    BatchKernel kern = batch_kernel(b->collision, b->storage, all_trim(b));
+    const bool fuse = b->storage == LBM_F32 && K >= kFuseMinK;
+    BatchKernel kern = batch_kernel(b->collision, b->storage, fuse, all_trim(b));
     int dev = 0, sms = 0, per_sm = 0;
     B_CUDA(b, cudaGetDevice(&dev));
     B_CUDA(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const size_t smem = b->storage == LBM_F32 ? TileGeo<kFuseX, kFuseY, kFuseSteps>::elems() * sizeof(float) : 0;
+    const size_t smem = fuse ? TileGeo<kFuseX, kFuseY, kFuseSteps>::elems() * sizeof(float) : 0;
     static_assert(TileGeo<kFuseX, kFuseY, kFuseSteps>::elems() * sizeof(float) <= 48 * 1024 - 256, "default shared memory");
     B_CUDA(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, b->block, smem));
     if (per_sm < 1) return bfail(b, LBM_ERR_ARG, "batch block size does not fit on an SM");
